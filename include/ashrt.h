@@ -153,7 +153,7 @@ ashrt_status ashrt_adjoint(const ashrt_plan* plan, const float* d_dev, float* m_
  * synchronise the device.  Computes what ashrt_forward computes for a plan
  * with the same arguments: the same tables and kernels, with the row kernel
  * in its radix-8 form (a plan's variant 3; a plan's default for Nt 1024..4096
- * is the radix-16 forward, which agrees with it to rounding).
+ * is a radix-16 forward, which agrees with it to rounding).
  *   nt, nx, dt, dx, velocities/nv, t0_shifts/nt0, opts: as ashrt_plan_create
  *     (apex positions are the trace positions; opts->max_batch and
  *     opts->with_solver are ignored)
@@ -338,8 +338,10 @@ ashrt_status ashrt_sort_gathers(const float* src_dev, int n0, int n1, int nt, fl
  * staged), 7: that forward with the radix-8 pair adjoint, 8: the radix-16
  * pair forward with that adjoint, 9: as 5 with the forward's per-bin sums in
  * tensor memory instead of registers (Nt = 2048 only, four CTAs per SM
- * instead of three; on other lengths the same kernels as 5); the default is 9
- * at Nt = 2048, 4 at Nt = 1024 and 4096, else 3)
+ * instead of three; on other lengths the same kernels as 5); without a set or
+ * tuned variant each call takes the form measured fastest for its batch: 3 up
+ * to Nt = 512, 6 at Nt = 1024 and 4096 and for small batches at Nt = 2048, 9 for
+ * large ones there, and between them the forward of 9 with the adjoint of 6)
  * and the trace-axis FFT column tile (16 or 8 columns for Nx <= 512) -- and
  * keeps the fastest in the plan; the plan's current choice is timed first and
  * another one replaces it only when it is more than 2% faster, so variants

@@ -5,6 +5,7 @@
 // in a JSON-lines cache keyed by device and problem shape.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -74,7 +75,7 @@ extern "C" ashrt_status ashrt_plan_autotune(ashrt_plan* p, int batch, const char
     return ASHRT_EINVAL;
   }
   const std::string key = tune_key(p, batch);
-  int minb = p->rows_minb, cols = p->xfft_cols;
+  int minb = 0, cols = p->xfft_cols;
   if (cache_lookup(cache_path, key, &minb, &cols)) {
     p->rows_minb = minb;
     p->xfft_cols = cols;
@@ -125,7 +126,8 @@ extern "C" ashrt_status ashrt_plan_autotune(ashrt_plan* p, int batch, const char
 
   // the plan's default variant is timed first and kept unless another one is
   // faster by more than 2% (timing noise does not flip the choice)
-  const int def_minb = p->rows_minb;
+  // (the rule's mixed form 10 is not a choice of its own: 9 stands for it)
+  const int def_minb = std::min(9, rows_variant(p, batch));
   std::vector<int> minbs = {def_minb};
   std::vector<int> cand = {3};
   if (p->logNt >= 9 && p->logNt <= 11) cand = {3, 2, 1};

@@ -81,13 +81,16 @@ struct RowArgs {
   int atab_ld = 0;                 // entries per (v, l) row: Nt/2 + 1 rounded up to 2
   const float2* phase = nullptr;   // [nt0][Nt] exp(-i w tau0), or null (tau0 == 0)
   int batch = 0;
+  int psplit = 1;                  // panel chunks a row's panels are split into (see
+                                   // rows_split); set by the launchers
   int minb = 3;                    // variant: 1, 2, 3 radix-8 kernels capped for that many
                                    // resident CTAs per SM; 4 radix-16 forward, radix-8
                                    // adjoint; 5 radix-16 both; 6 single-gather radix-16
                                    // both; 7 single-gather radix-16 forward, radix-8
                                    // adjoint; 8 radix-16 pair forward, single-gather
                                    // radix-16 adjoint; 9 as 5 with the forward's
-                                   // accumulator in tensor memory (4..9 need tw16)
+                                   // accumulator in tensor memory; 10 the forward of 9 with
+                                   // the adjoint of 6 (4..10 need tw16)
 };
 
 cudaError_t launch_xfft_r2c(const XfftArgs& a, cudaStream_t s);
@@ -194,7 +197,8 @@ struct ashrt_plan {
   int with_solver = 0;
   ashrt_opts opts{};
   bool shift = false;        // any nonzero tau0
-  int rows_minb = 3;         // row-kernel variant 1..9 (autotuned; see ashrt_plan_autotune)
+  int rows_minb = 3;         // row-kernel variant 1..9 (set or autotuned; see
+                             // ashrt_plan_autotune), 0: by rule (rows_variant)
   int xfft_cols = 16;
   // device tables
   float2* tw_t = nullptr;

@@ -14,6 +14,9 @@ constexpr int kSelStride = 2048;
 size_t model_elems(const ashrt_plan* p);
 size_t data_elems(const ashrt_plan* p);
 
+// The row-kernel variant of a call (the plan's, or by rule for its sizes).
+int rows_variant(const ashrt_plan* p, int batch);
+
 // cg (optional): a CGLS update fused into the operator's first transform, on
 // the input m (forward, mode 1) or d (adjoint, mode 2), which is then written.
 cudaError_t op_forward(const ashrt_plan* p, const float* m, float* d, const float* ew_model,

@@ -172,6 +172,27 @@ static ashrt_status upload(T** ptr, const std::vector<T>& host, size_t* total) {
 size_t model_elems(const ashrt_plan* p) { return (size_t)p->P * p->nx * p->nt; }
 size_t data_elems(const ashrt_plan* p) { return (size_t)p->nr * p->nt; }
 
+// The row kernels' form for a batch when none was set or tuned, from both
+// sides measured (us per launch, forward / adjoint; R = batch x (Nx/2 + 1) rows):
+//   Nt <= 512: the radix-8 pair kernels (the only ones).
+//   Nt 4096: the single-gather form (6) at every batch: a pair fills an SM's
+//     shared memory with one or two CTAs of 8 warps.  24 panels, 513 rows:
+//     5 gathers 693 / 732 against 946 / 1040 (4), 32 gathers 4353 / 4540
+//     against 4790 / 5258.
+//   Nt 1024: the single-gather form: 16 panels, 129 rows, 16 gathers 95 / 94
+//     against 121 / 111 (4), 64 gathers 347 / 338 against 336 / 369.
+//   Nt 2048, 32 panels, 257 rows: the pair form (9) shares each twiddle and
+//     table read between two gathers, which wins once pairs alone fill the
+//     chip: forward 3 gathers (R = 771) 158 single against 175, 4 (1028) 191
+//     against 179; adjoint 12 gathers (3084) 511 against 518, 64 gathers 2593
+//     against 2491.  So single below R = 900 (forward) and 3600 (adjoint).
+int rows_variant(const ashrt_plan* p, int batch) {
+  if (p->rows_minb) return p->rows_minb;
+  if (p->logNt != 11) return 6;
+  const long long R = (long long)batch * p->Lh;
+  return R <= 900 ? 6 : (R <= 3600 ? 10 : 9);
+}
+
 // ---------------------------------------------------------------------------
 // Operator application with the fused IRLS weights.
 //   forward: d = tmask * ew_data * L(ew_model * m); dot[g] += ||d_g||^2
@@ -232,7 +253,7 @@ cudaError_t op_forward(const ashrt_plan* p, const float* m, float* d, const floa
   ra.taps_ld = taps_row_len(p->Nt);
   ra.phase = p->shift ? p->phase : nullptr;
   ra.batch = batch;
-  ra.minb = p->rows_minb;
+  ra.minb = rows_variant(p, batch);
   prof_begin(PROF_ROWS_FWD, s);
   e = launch_stolt_fwd_rows(ra, s);
   prof_end(PROF_ROWS_FWD, s);
@@ -327,7 +348,7 @@ cudaError_t op_adjoint(const ashrt_plan* p, const float* d, float* m, const floa
   ra.atab_ld = atab_row_len(p->Nt);
   ra.phase = p->shift ? p->phase : nullptr;
   ra.batch = batch;
-  ra.minb = p->rows_minb;
+  ra.minb = rows_variant(p, batch);
   prof_begin(PROF_ROWS_ADJ, s);
   e = launch_stolt_adj_rows(ra, s);
   prof_end(PROF_ROWS_ADJ, s);
@@ -534,10 +555,7 @@ static ashrt_status plan_create_impl(ashrt_plan** out, int nt, int nx, double dt
     std::vector<float2> tw16(twiddle_table_len(p->logNt, 4));
     build_twiddle_table(p->logNt, tw16.data(), 4);
     chk(upload(&p->tw_t16, tw16, &total));
-    // the fastest pair measured: at Nt = 2048 radix-16 both ways with the
-    // forward's accumulator in tensor memory, elsewhere radix-16 forward and
-    // radix-8 adjoint
-    p->rows_minb = p->logNt == 11 ? 9 : 4;
+    p->rows_minb = 0;   // by rule (rows_variant) until a variant is set or tuned
   }
   chk(upload(&p->wt, wt, &total));
   chk(upload(&p->kmin, kmin, &total));

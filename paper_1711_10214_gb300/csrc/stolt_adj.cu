@@ -46,7 +46,8 @@ namespace {
 // taken from the tap words; see build_adj_table) staged per panel gives them
 // directly.  Every output bin is written once, by its owner: no atomics, no
 // clearing pass, no search, and the strided ownership spreads the bins
-// outside the cone over all warps.
+// outside the cone over all warps.  The grid's z splits the panels into
+// chunks, each CTA transforming the data rows for its own.
 template <int LOGN, bool SHIFT, int MINB, bool HALF>
 __global__ void __launch_bounds__((1 << LOGN) / 8, MINB)
 stolt_adj_rows(RowArgs a) {
@@ -61,7 +62,11 @@ stolt_adj_rows(RowArgs a) {
   const float2* yA = a.Y + (long long)b0 * a.y_batch + (long long)l * a.ld;
   const uint2* arow = a.atab + (long long)l * a.atab_ld;
   const long long astep = (long long)a.Lh * a.atab_ld;
-  stage_tab(stab, arow, a.atab_ld, tid, T);
+  int p0, p1;
+  panel_chunk(a.P, gridDim.z, blockIdx.z, p0, p1);
+  if (p0 >= p1) return;
+  int iv = p0 % a.nv, jt = p0 / a.nv;
+  stage_tab(stab, arow + iv * astep, a.atab_ld, tid, T);
   cp_async_commit();
 
   float4 v[8];
@@ -76,14 +81,13 @@ stolt_adj_rows(RowArgs a) {
 
   float2* xA = a.Xw + (long long)b0 * a.x_batch + (long long)l * a.ld;
   float2* xB = hasB ? xA + a.x_batch : nullptr;
-  int iv = 0, jt = 0;
-  int km = __ldg(a.kmin + l);                   // cone start of the panel's (velocity, k_x)
-  for (int p = 0; p < a.P; ++p) {
+  int km = __ldg(a.kmin + iv * a.Lh + l);       // cone start of the panel's (velocity, k_x)
+  for (int p = p0; p < p1; ++p) {
     cp_async_wait_all();
     __syncthreads();
     const bool mapped = km < H;
     // the next panel's, loaded a panel ahead of its use
-    if (p + 1 < a.P) km = __ldg(a.kmin + (iv + 1 == a.nv ? 0 : iv + 1) * a.Lh + l);
+    if (p + 1 < p1) km = __ldg(a.kmin + (iv + 1 == a.nv ? 0 : iv + 1) * a.Lh + l);
     const float2* phj = SHIFT ? a.phase + (long long)jt * N : nullptr;
     // the bins this thread gathers, j = tid + T s, are exactly the inputs of
     // its first inverse-FFT butterfly: they stay in registers
@@ -96,7 +100,7 @@ stolt_adj_rows(RowArgs a) {
     // first pass from the registers (its barrier also ends every thread's
     // reads of the source-table row, which is then restaged)
     row_first_pass<+1, N>(buf, accs, tid);
-    if (p + 1 < a.P) {
+    if (p + 1 < p1) {
       const int ivn = iv + 1 == a.nv ? 0 : iv + 1;
       stage_tab(stab, arow + ivn * astep, a.atab_ld, tid, T);
       cp_async_commit();
@@ -120,7 +124,10 @@ cudaError_t launch_adj_vh(const RowArgs& a, cudaStream_t s) {
   const size_t smem = (size_t)2 * N * sizeof(float4) + (size_t)a.atab_ld * sizeof(uint2);
   cudaError_t e = set_smem(stolt_adj_rows<LOGN, SHIFT, MINB, HALF>, smem_cap<LOGN>(false), attr);
   if (e != cudaSuccess) return e;
-  stolt_adj_rows<LOGN, SHIFT, MINB, HALF><<<dim3(a.Lh, (a.batch + 1) / 2), N / 8, smem, s>>>(a);
+  // rows of Nt <= 512 may fill an SM with more than MINB CTAs
+  const int n = rows_split((long long)a.Lh * ((a.batch + 1) / 2), a.P, LOGN <= 9 ? 8 : MINB);
+  stolt_adj_rows<LOGN, SHIFT, MINB, HALF>
+      <<<dim3(a.Lh, (a.batch + 1) / 2, n), N / 8, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -157,10 +164,10 @@ cudaError_t launch_adj_t(const RowArgs& a, cudaStream_t s) {
 
 // Variants (a.minb): 1..3 radix-8 with that register cap; 4 and 7 radix-8
 // cap 3 (the forward alone is radix-16); 5 and 9 the radix-16 pair adjoint
-// (stolt_r16.cu), 6 and 8 the single-gather radix-16 adjoint (stolt_r16s.cu)
+// (stolt_r16.cu), 6, 8 and 10 the single-gather radix-16 adjoint (stolt_r16s.cu)
 // where their twiddles exist, else cap 3.
 cudaError_t launch_stolt_adj_rows(const RowArgs& a, cudaStream_t s) {
-  if ((a.minb == 6 || a.minb == 8) && a.tw16) return launch_stolt_adj_rows16s(a, s);
+  if ((a.minb == 6 || a.minb == 8 || a.minb == 10) && a.tw16) return launch_stolt_adj_rows16s(a, s);
   if ((a.minb == 5 || a.minb == 9) && a.tw16) return launch_stolt_adj_rows16(a, s);
   RowArgs b = a;
   if (b.minb > 3) b.minb = 3;

@@ -30,6 +30,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -207,6 +209,123 @@ inline int row_log2(int n) {
   int l = 0;
   while ((1 << l) < n) ++l;
   return l;
+}
+
+// The panels [p0, p1) of chunk z when P panels are split into n chunks.
+__device__ __forceinline__ void panel_chunk(int P, int n, int z, int& p0, int& p1) {
+  const int per = (P + n - 1) / n;
+  p0 = min(P, z * per);
+  p1 = min(P, p0 + per);
+}
+
+// Chunks a row's panels are split into, so that few rows (small batches,
+// narrow gathers) still fill the chip: 1, 2, 4 or 8.  `ctas` rows of P panels
+// each run as ctas x n CTAs, `res` of them resident per SM.  A panel takes a
+// CTA about a + b k with k CTAs on its SM (a: the latency of its dependent
+// passes, b: its share of the shared-memory pipe; a/b about 2.5 in all the row
+// kernels: e.g. the single-gather forward at Nt 2048 1.2 us and 0.5 us), and
+// every chunk costs about one and a half panels more (setup and the extra
+// data-row transform of the adjoint, or the sum over the chunks of the
+// forward), so the candidate with the smallest
+//   waves(n) (P / n + 1.5) (2.5 + k(n))
+// is taken.  Forward / adjoint rows per launch, before and after: 1 gather
+// 256 x 64, 8 panels (65 rows) 16.3 / 18.2 -> 11.8 / 10.3 us; 2 gathers
+// 181 x 455, 25 panels (513 rows of pairs) 51 / 54 -> 43 / 41 us; 1 gather
+// 1024 x 256, 32 panels (257 rows, single-gather form) 75 / 82 -> 62 / 60 us;
+// 2 gathers 1024 x 128, 192 panels (258 rows) 451 / 555 -> 349 / 347 us.
+inline int rows_split(long long ctas, int P, int res) {
+  constexpr int kSms = 152;
+  int best = 1;
+  double best_t = 0.0;
+  for (int n = 1; n <= 8 && (n == 1 || n <= P); n *= 2) {
+    const double per_sm = (double)((ctas * n + kSms - 1) / kSms);
+    const double k = per_sm < res ? per_sm : res;
+    const double waves = std::ceil(per_sm / k);
+    const double t = waves * ((P + n - 1) / n + 1.5) * (2.5 + k);
+    if (n == 1 || t < 0.95 * best_t) {
+      best = n;
+      best_t = t;
+    }
+  }
+  return best;
+}
+
+// Barrier of the thread-block cluster (all threads of all its CTAs).
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
+  return r;
+}
+// 16 or 8 bytes of the same shared variable in the CTA of rank `rank`.
+__device__ __forceinline__ unsigned cluster_addr(const void* p, unsigned rank) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n"
+               : "=r"(r)
+               : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_load(unsigned a, float4& v) {
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(a)
+               : "memory");
+}
+__device__ __forceinline__ void cluster_load(unsigned a, float2& v) {
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];\n"
+               : "=f"(v.x), "=f"(v.y)
+               : "r"(a)
+               : "memory");
+}
+
+// The forward's sum over the panel chunks of a row: the chunks' CTAs are one
+// cluster, each leaves its V bins per thread (k = tid + T s) in its own shared
+// row, and rank 0 adds them in rank order (the sum does not depend on the
+// scheduling).  Returns false in the other ranks, which are then done.
+template <int V, int T, typename E>
+__device__ __forceinline__ bool cluster_sum_rows(E* buf, E* acc, int tid, int n) {
+  const unsigned rank = cluster_rank();
+  __syncthreads();
+  if (rank != 0) {
+#pragma unroll
+    for (int s = 0; s < V; ++s) buf[tid + T * s] = acc[s];
+  }
+  cluster_barrier();
+  if (rank == 0) {
+    for (int r = 1; r < n; ++r) {
+      const unsigned a = cluster_addr(buf, r);
+#pragma unroll
+      for (int s = 0; s < V; ++s) {
+        E v;
+        cluster_load(a + (unsigned)((tid + T * s) * sizeof(E)), v);
+        acc[s] = cadd(acc[s], v);
+      }
+    }
+  }
+  cluster_barrier();   // a CTA's shared memory lives until rank 0 has read it
+  return rank == 0;
+}
+
+// Launch of a row kernel whose grid's z dimension is one cluster of n CTAs.
+template <typename K>
+inline cudaError_t launch_cluster_z(K kern, dim3 grid, int threads, size_t smem, int n,
+                                    cudaStream_t s, const RowArgs& a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 1;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = n;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
 }  // namespace ashrt

@@ -39,8 +39,11 @@ namespace {
 // are interleaved element by element, so every shared access is 16 bytes and
 // the twiddles and Stolt taps are computed once for both gathers.
 // HALF: nt <= Nt / 2, so inputs tid + r Nt/8 with r >= 4 are zero padding.
-template <int LOGN, bool SHIFT, int MINB, bool HALF>
-__global__ void __launch_bounds__((1 << LOGN) / 8, MINB)
+// SPLIT: the panels are split over the CTAs of a cluster along the grid's z
+// (register cap for eight resident CTAs: without it the sum over the chunks
+// takes 168 registers and a split grid no longer fits in one wave).
+template <int LOGN, bool SHIFT, int MINB, bool HALF, bool SPLIT>
+__global__ void __launch_bounds__((1 << LOGN) / 8, SPLIT ? 8 : MINB)
 stolt_fwd_rows(RowArgs a) {
   constexpr int N = 1 << LOGN, T = N / 8;
   using S = Sched<LOGN>;
@@ -63,12 +66,17 @@ stolt_fwd_rows(RowArgs a) {
   }
   const unsigned* trow = a.taps + (long long)l * a.taps_ld;   // velocity iv: + iv * Lh * taps_ld
   const long long tstep = (long long)a.Lh * a.taps_ld;
-  stage_rows(stage, xA, xB, a.ld, tid, T);
-  stage_taps(stap0, trow, a.taps_ld, tid, T);
+  int p0 = 0, p1 = a.P;
+  if (SPLIT) panel_chunk(a.P, a.psplit, blockIdx.z, p0, p1);
+  int iv = SPLIT ? p0 % a.nv : 0, jt = SPLIT ? p0 / a.nv : 0;
+  if (!SPLIT || p0 < p1) {
+    const long long o = (long long)p0 * a.x_panel;
+    stage_rows(stage, xA + o, hasB ? xB + o : nullptr, a.ld, tid, T);
+    stage_taps((p0 & 1) ? stap1 : stap0, trow + iv * tstep, a.taps_ld, tid, T);
+  }
   cp_async_commit();
 
-  int iv = 0, jt = 0;
-  for (int p = 0; p < a.P; ++p) {
+  for (int p = p0; p < p1; ++p) {
     unsigned* stap = (p & 1) ? stap1 : stap0;
     cp_async_wait_all();
     __syncthreads();
@@ -85,14 +93,14 @@ stolt_fwd_rows(RowArgs a) {
       v[r] = pack2(za, zb);
     }
     __syncthreads();
-    if (p + 1 < a.P) {
+    if (p + 1 < p1) {
       const long long o = (long long)(p + 1) * a.x_panel;
       const int ivn = iv + 1 == a.nv ? 0 : iv + 1;
       stage_rows(stage, xA + o, hasB ? xB + o : nullptr, a.ld, tid, T);
       stage_taps((p & 1) ? stap0 : stap1, trow + ivn * tstep, a.taps_ld, tid, T);
       cp_async_commit();
     }
-    if (SHIFT && iv == 0) {
+    if (SHIFT && (iv == 0 || (SPLIT && p == p0))) {
 #pragma unroll
       for (int s = 0; s < 8; ++s) ph[s] = __ldg(a.phase + (long long)jt * N + tid + T * s);
     }
@@ -117,6 +125,7 @@ stolt_fwd_rows(RowArgs a) {
     }
     __syncthreads();
   }
+  if (SPLIT && !cluster_sum_rows<8, T>(buf, acc, tid, a.psplit)) return;
 #pragma unroll
   for (int s = 0; s < 8; ++s) acc[s] = cscale(acc[s], __ldg(a.wt + tid + T * s));
   // own bins are exactly the first-pass inputs of the inverse transform
@@ -129,14 +138,29 @@ stolt_fwd_rows(RowArgs a) {
 
 
 template <int LOGN, bool SHIFT, int MINB, bool HALF>
-cudaError_t launch_fwd_vh(const RowArgs& a, cudaStream_t s) {
+cudaError_t launch_fwd_vh(const RowArgs& a0, cudaStream_t s) {
   constexpr int N = 1 << LOGN;
-  static bool attr = false;
+  RowArgs a = a0;
   const size_t smem = (size_t)N * sizeof(float4) + (size_t)2 * a.ld * sizeof(float2) +
                       (size_t)2 * a.taps_ld * sizeof(unsigned);
-  cudaError_t e = set_smem(stolt_fwd_rows<LOGN, SHIFT, MINB, HALF>, smem_cap<LOGN>(true), attr);
+  const dim3 grid(a.Lh, (a.batch + 1) / 2);
+  if constexpr (LOGN <= 9) {
+    // longer rows have single-gather kernels for batches this small
+    a.psplit = rows_split((long long)grid.x * grid.y, a.P, 8);
+    if (a.psplit > 1) {
+      static bool attr = false;
+      cudaError_t e = set_smem(stolt_fwd_rows<LOGN, SHIFT, MINB, HALF, true>, smem_cap<LOGN>(true),
+                               attr);
+      if (e != cudaSuccess) return e;
+      return launch_cluster_z(stolt_fwd_rows<LOGN, SHIFT, MINB, HALF, true>,
+                              dim3(grid.x, grid.y, a.psplit), N / 8, smem, a.psplit, s, a);
+    }
+  }
+  static bool attr = false;
+  cudaError_t e = set_smem(stolt_fwd_rows<LOGN, SHIFT, MINB, HALF, false>, smem_cap<LOGN>(true),
+                           attr);
   if (e != cudaSuccess) return e;
-  stolt_fwd_rows<LOGN, SHIFT, MINB, HALF><<<dim3(a.Lh, (a.batch + 1) / 2), N / 8, smem, s>>>(a);
+  stolt_fwd_rows<LOGN, SHIFT, MINB, HALF, false><<<grid, N / 8, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -170,12 +194,12 @@ cudaError_t launch_fwd_t(const RowArgs& a, cudaStream_t s) {
 }  // namespace
 
 // Variants (a.minb): 1..3 radix-8 with that register cap; 4, 5 and 8 use the
-// radix-16 pair forward (stolt_r16.cu), 9 its tensor-memory-accumulator form
+// radix-16 pair forward (stolt_r16.cu), 9 and 10 its tensor-memory-accumulator form
 // (Nt = 2048; the register form elsewhere), 6 and 7 the single-gather radix-16
 // forward (stolt_r16s.cu) where their twiddles exist, else cap 3.
 cudaError_t launch_stolt_fwd_rows(const RowArgs& a, cudaStream_t s) {
   if ((a.minb == 6 || a.minb == 7) && a.tw16) return launch_stolt_fwd_rows16s(a, s);
-  if (a.minb == 9 && a.tw16) return launch_stolt_fwd_rows16_tm(a, s);
+  if ((a.minb == 9 || a.minb == 10) && a.tw16) return launch_stolt_fwd_rows16_tm(a, s);
   if (a.minb >= 4 && a.tw16) return launch_stolt_fwd_rows16(a, s);
   RowArgs b = a;
   if (b.minb > 3) b.minb = 3;

@@ -74,7 +74,8 @@ __device__ __forceinline__ float2 adj_gather1(const float2* dsp, uint2 e, int j,
 // row, FFT it along tau, and accumulate the interpolated bins of the Stolt
 // map (taps from the tap word of |k|) times the asymptote phase in registers;
 // finally weight by W(w) / (Nt Nx), inverse FFT, keep nt samples.
-template <int LOGN, bool SHIFT, bool HALF>
+// SPLIT: the panels are split over the CTAs of a cluster along the grid's z.
+template <int LOGN, bool SHIFT, bool HALF, bool SPLIT>
 __global__ void __launch_bounds__((1 << LOGN) / 16, r16s_minb_fwd<LOGN>())
 stolt_fwd_rows16s(RowArgs a) {
   constexpr int N = 1 << LOGN, T = N / 16;
@@ -90,11 +91,13 @@ stolt_fwd_rows16s(RowArgs a) {
   for (int s = 0; s < 16; ++s) acc[s] = make_float2(0.f, 0.f);
   const unsigned* trow = a.taps + (long long)l * a.taps_ld;
   const long long tstep = (long long)a.Lh * a.taps_ld;
-  stage_row1(stage, xr, a.ld, tid, T);
+  int p0 = 0, p1 = a.P;
+  if (SPLIT) panel_chunk(a.P, a.psplit, blockIdx.z, p0, p1);
+  if (!SPLIT || p0 < p1) stage_row1(stage, xr + (long long)p0 * a.x_panel, a.ld, tid, T);
   cp_async_commit();
 
-  int iv = 0, jt = 0;
-  for (int p = 0; p < a.P; ++p) {
+  int iv = SPLIT ? p0 % a.nv : 0, jt = SPLIT ? p0 / a.nv : 0;
+  for (int p = p0; p < p1; ++p) {
     // this panel's tap words, consumed after the transform
     unsigned tw[16];
     const unsigned* tr = trow + iv * tstep;
@@ -109,7 +112,7 @@ stolt_fwd_rows16s(RowArgs a) {
       v[r] = (!(HALF && r >= 8) && i < a.nt) ? stage[i] : make_float2(0.f, 0.f);
     }
     __syncthreads();
-    if (p + 1 < a.P) {
+    if (p + 1 < p1) {
       stage_row1(stage, xr + (long long)(p + 1) * a.x_panel, a.ld, tid, T);
       cp_async_commit();
     }
@@ -132,12 +135,13 @@ stolt_fwd_rows16s(RowArgs a) {
     }
     __syncthreads();
   }
+  if (SPLIT && !cluster_sum_rows<16, T>(buf, acc, tid, a.psplit)) return;
 #pragma unroll
   for (int s = 0; s < 16; ++s) acc[s] = cscale(acc[s], __ldg(a.wt + tid + T * s));
   // own bins are exactly the first-pass inputs of the inverse transform
   r16_first_pass<+1>(buf, acc, tid);
   r16_pass_range<+1, LOGN, 1, S::NPASS - 1>(buf, a.tw16, tid);
-  r16_last_pass_global<+1, LOGN>(buf, a.tw16, tid,
+  r16_last_pass_global<+1, LOGN, float2, HALF>(buf, a.tw16, tid,
                                  a.Yw + (long long)b * a.y_batch + (long long)l * a.ld, nullptr,
                                  a.nt);
 }
@@ -146,8 +150,10 @@ stolt_fwd_rows16s(RowArgs a) {
 // every panel gather each output bin j = tid + T s from its at most two
 // sources (source-table entry of |j|, loaded one panel ahead), inverse FFT,
 // keep nt samples.  A (velocity, k_x) row entirely outside the cone gives a
-// zero panel row without a transform.
-template <int LOGN, bool SHIFT>
+// zero panel row without a transform.  The grid's z splits the panels into
+// chunks, each CTA transforming the data row for its own.  HALF: nt <= Nt / 2,
+// so only the lower half of each inverse transform is formed.
+template <int LOGN, bool SHIFT, bool HALF>
 __global__ void __launch_bounds__((1 << LOGN) / 16, r16s_minb_adj<LOGN>())
 stolt_adj_rows16s(RowArgs a) {
   constexpr int N = 1 << LOGN, T = N / 16, H = N / 2;
@@ -160,9 +166,15 @@ stolt_adj_rows16s(RowArgs a) {
   const uint2* arow = a.atab + (long long)l * a.atab_ld;
   const long long astep = (long long)a.Lh * a.atab_ld;
 
+  int p0, p1;
+  panel_chunk(a.P, gridDim.z, blockIdx.z, p0, p1);
+  if (p0 >= p1) return;
+  int iv = p0 % a.nv, jt = p0 / a.nv;
+
   uint2 ent[16];
 #pragma unroll
-  for (int s = 0; s < 16; ++s) ent[s] = __ldg(arow + kabs_of<N>(tid + T * s));
+  for (int s = 0; s < 16; ++s)
+    ent[s] = __ldg(arow + iv * astep + kabs_of<N>(tid + T * s));
   {
     float2 v[16];
 #pragma unroll
@@ -180,14 +192,13 @@ stolt_adj_rows16s(RowArgs a) {
   }
 
   float2* xr = a.Xw + (long long)b * a.x_batch + (long long)l * a.ld;
-  int iv = 0, jt = 0;
-  int km = __ldg(a.kmin + l);                   // cone start of the panel's (velocity, k_x)
-  for (int p = 0; p < a.P; ++p) {
+  int km = __ldg(a.kmin + iv * a.Lh + l);       // cone start of the panel's (velocity, k_x)
+  for (int p = p0; p < p1; ++p) {
     // dsp complete (first panel); the previous panel's reads of buf done
     __syncthreads();
     const long long o = (long long)p * a.x_panel;
     const int ivn = iv + 1 == a.nv ? 0 : iv + 1;
-    const bool more = p + 1 < a.P;
+    const bool more = p + 1 < p1;
     const bool unmapped = km >= H;
     if (more) km = __ldg(a.kmin + ivn * a.Lh + l);   // the next panel's, a panel ahead
     if (unmapped) {
@@ -215,7 +226,7 @@ stolt_adj_rows16s(RowArgs a) {
       }
       r16_first_pass<+1>(buf, accs, tid);
       r16_pass_range<+1, LOGN, 1, S::NPASS - 1>(buf, a.tw16, tid);
-      r16_last_pass_global<+1, LOGN>(buf, a.tw16, tid, xr + o, nullptr, a.nt);
+      r16_last_pass_global<+1, LOGN, float2, HALF>(buf, a.tw16, tid, xr + o, nullptr, a.nt);
     }
     iv = ivn;
     if (iv == 0) ++jt;
@@ -223,14 +234,22 @@ stolt_adj_rows16s(RowArgs a) {
 }
 
 template <int LOGN, bool SHIFT, bool HALF>
-cudaError_t launch_fwd16s_h(const RowArgs& a, cudaStream_t s) {
+cudaError_t launch_fwd16s_h(const RowArgs& a0, cudaStream_t s) {
   constexpr int N = 1 << LOGN;
+  RowArgs a = a0;
+  a.psplit = rows_split((long long)a.batch * a.Lh, a.P, r16s_minb_fwd<LOGN>());
+  const size_t smem = (size_t)(N + a.ld) * sizeof(float2), cap = (size_t)2 * N * sizeof(float2);
+  if (a.psplit > 1) {
+    static bool attr = false;
+    cudaError_t e = set_smem(stolt_fwd_rows16s<LOGN, SHIFT, HALF, true>, cap, attr);
+    if (e != cudaSuccess) return e;
+    return launch_cluster_z(stolt_fwd_rows16s<LOGN, SHIFT, HALF, true>,
+                            dim3(a.batch, a.Lh, a.psplit), N / 16, smem, a.psplit, s, a);
+  }
   static bool attr = false;
-  const size_t smem = (size_t)(N + a.ld) * sizeof(float2);
-  cudaError_t e = set_smem(stolt_fwd_rows16s<LOGN, SHIFT, HALF>, (size_t)2 * N * sizeof(float2),
-                           attr);
+  cudaError_t e = set_smem(stolt_fwd_rows16s<LOGN, SHIFT, HALF, false>, cap, attr);
   if (e != cudaSuccess) return e;
-  stolt_fwd_rows16s<LOGN, SHIFT, HALF><<<dim3(a.batch, a.Lh), N / 16, smem, s>>>(a);
+  stolt_fwd_rows16s<LOGN, SHIFT, HALF, false><<<dim3(a.batch, a.Lh), N / 16, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -240,15 +259,22 @@ cudaError_t launch_fwd16s(const RowArgs& a, cudaStream_t s) {
                           : launch_fwd16s_h<LOGN, SHIFT, false>(a, s);
 }
 
-template <int LOGN, bool SHIFT>
-cudaError_t launch_adj16s(const RowArgs& a, cudaStream_t s) {
+template <int LOGN, bool SHIFT, bool HALF>
+cudaError_t launch_adj16s_h(const RowArgs& a, cudaStream_t s) {
   constexpr int N = 1 << LOGN;
   static bool attr = false;
   const size_t smem = (size_t)2 * N * sizeof(float2);
-  cudaError_t e = set_smem(stolt_adj_rows16s<LOGN, SHIFT>, smem, attr);
+  cudaError_t e = set_smem(stolt_adj_rows16s<LOGN, SHIFT, HALF>, smem, attr);
   if (e != cudaSuccess) return e;
-  stolt_adj_rows16s<LOGN, SHIFT><<<dim3(a.batch, a.Lh), N / 16, smem, s>>>(a);
+  const int n = rows_split((long long)a.batch * a.Lh, a.P, r16s_minb_adj<LOGN>());
+  stolt_adj_rows16s<LOGN, SHIFT, HALF><<<dim3(a.batch, a.Lh, n), N / 16, smem, s>>>(a);
   return cudaGetLastError();
+}
+
+template <int LOGN, bool SHIFT>
+cudaError_t launch_adj16s(const RowArgs& a, cudaStream_t s) {
+  return 2 * a.nt <= a.Nt ? launch_adj16s_h<LOGN, SHIFT, true>(a, s)
+                          : launch_adj16s_h<LOGN, SHIFT, false>(a, s);
 }
 
 }  // namespace
