@@ -125,7 +125,8 @@ cudaError_t launch_adj_vh(const RowArgs& a, cudaStream_t s) {
   cudaError_t e = set_smem(stolt_adj_rows<LOGN, SHIFT, MINB, HALF>, smem_cap<LOGN>(false), attr);
   if (e != cudaSuccess) return e;
   // rows of Nt <= 512 may fill an SM with more than MINB CTAs
-  const int n = rows_split((long long)a.Lh * ((a.batch + 1) / 2), a.P, LOGN <= 9 ? 8 : MINB);
+  const int n = rows_split((long long)a.Lh * ((a.batch + 1) / 2), a.P, LOGN <= 9 ? 8 : MINB,
+                           false);
   stolt_adj_rows<LOGN, SHIFT, MINB, HALF>
       <<<dim3(a.Lh, (a.batch + 1) / 2, n), N / 8, smem, s>>>(a);
   return cudaGetLastError();

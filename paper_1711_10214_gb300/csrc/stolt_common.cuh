@@ -228,16 +228,19 @@ __device__ __forceinline__ void panel_chunk(int P, int n, int z, int& p0, int& p
 // data-row transform of the adjoint, or the sum over the chunks of the
 // forward), so the candidate with the smallest
 //   waves(n) (P / n + 1.5) (2.5 + k(n))
-// is taken.  Forward / adjoint rows per launch, before and after: 1 gather
-// 256 x 64, 8 panels (65 rows) 16.3 / 18.2 -> 11.8 / 10.3 us; 2 gathers
-// 181 x 455, 25 panels (513 rows of pairs) 51 / 54 -> 43 / 41 us; 1 gather
+// is taken.  `ordered` (the forward): up to eight panels are split one to a
+// CTA or not at all, so that the partial sums, added in rank order, are those
+// of the unsplit loop to the last bit.  Forward / adjoint rows per launch, before and after: 1 gather
+// 256 x 64, 8 panels (65 rows) 16.3 / 18.2 -> 11.0 / 10.4 us; 2 gathers
+// 181 x 455, 25 panels (513 rows of pairs) 51 / 54 -> 45 / 41 us; 1 gather
 // 1024 x 256, 32 panels (257 rows, single-gather form) 75 / 82 -> 62 / 60 us;
 // 2 gathers 1024 x 128, 192 panels (258 rows) 451 / 555 -> 349 / 347 us.
-inline int rows_split(long long ctas, int P, int res) {
+inline int rows_split(long long ctas, int P, int res, bool ordered) {
   constexpr int kSms = 152;
   int best = 1;
   double best_t = 0.0;
-  for (int n = 1; n <= 8 && (n == 1 || n <= P); n *= 2) {
+  const bool whole = ordered && P <= 8;
+  for (int n = 1; n <= 8 && n <= P; n = whole && n < P ? P : 2 * n) {
     const double per_sm = (double)((ctas * n + kSms - 1) / kSms);
     const double k = per_sm < res ? per_sm : res;
     const double waves = std::ceil(per_sm / k);
@@ -281,38 +284,53 @@ __device__ __forceinline__ void cluster_load(unsigned a, float2& v) {
                : "memory");
 }
 
+__device__ __forceinline__ void cluster_store(unsigned a, float4 v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"r"(a), "f"(v.x), "f"(v.y),
+               "f"(v.z), "f"(v.w)
+               : "memory");
+}
+__device__ __forceinline__ void cluster_store(unsigned a, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};\n" ::"r"(a), "f"(v.x), "f"(v.y)
+               : "memory");
+}
+
 // The forward's sum over the panel chunks of a row: the chunks' CTAs are one
 // cluster, each leaves its V bins per thread (k = tid + T s) in its own shared
-// row, and rank 0 adds them in rank order (the sum does not depend on the
-// scheduling).  Returns false in the other ranks, which are then done.
+// row, and every CTA adds its share of the bins over all of them, in rank order
+// (the sum does not depend on the scheduling), into rank 0's row.  The n loads
+// of a bin are in flight together: rank 0 adding row after row takes 2.7 us
+// longer for eight chunks at Nt 512.  Returns false in the other ranks, which
+// are then done.
 template <int V, int T, typename E>
 __device__ __forceinline__ bool cluster_sum_rows(E* buf, E* acc, int tid, int n) {
   const unsigned rank = cluster_rank();
   __syncthreads();
-  if (rank != 0) {
 #pragma unroll
-    for (int s = 0; s < V; ++s) buf[tid + T * s] = acc[s];
-  }
+  for (int s = 0; s < V; ++s) buf[tid + T * s] = acc[s];
   cluster_barrier();
-  if (rank == 0) {
-    for (int r = 1; r < n; ++r) {
-      const unsigned a = cluster_addr(buf, r);
+  for (int k = (int)rank * T + tid; k < V * T; k += n * T) {
+    E v[8];
 #pragma unroll
-      for (int s = 0; s < V; ++s) {
-        E v;
-        cluster_load(a + (unsigned)((tid + T * s) * sizeof(E)), v);
-        acc[s] = cadd(acc[s], v);
-      }
-    }
+    for (int r = 0; r < 8; ++r)
+      if (r < n) cluster_load(cluster_addr(buf + k, r), v[r]);
+    E sum = v[0];
+#pragma unroll
+    for (int r = 1; r < 8; ++r)
+      if (r < n) sum = cadd(sum, v[r]);
+    cluster_store(cluster_addr(buf + k, 0), sum);
   }
-  cluster_barrier();   // a CTA's shared memory lives until rank 0 has read it
-  return rank == 0;
+  cluster_barrier();   // (also: a CTA's shared memory lives until the others have read it)
+  if (rank != 0) return false;
+#pragma unroll
+  for (int s = 0; s < V; ++s) acc[s] = buf[tid + T * s];
+  __syncthreads();     // every read of the row before the transform writes it
+  return true;
 }
 
-// Launch of a row kernel whose grid's z dimension is one cluster of n CTAs.
-template <typename K>
+// Launch of a kernel whose grid's z dimension is one cluster of n CTAs.
+template <typename K, typename A>
 inline cudaError_t launch_cluster_z(K kern, dim3 grid, int threads, size_t smem, int n,
-                                    cudaStream_t s, const RowArgs& a) {
+                                    cudaStream_t s, const A& a) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);

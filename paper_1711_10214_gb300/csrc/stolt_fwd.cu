@@ -146,7 +146,7 @@ cudaError_t launch_fwd_vh(const RowArgs& a0, cudaStream_t s) {
   const dim3 grid(a.Lh, (a.batch + 1) / 2);
   if constexpr (LOGN <= 9) {
     // longer rows have single-gather kernels for batches this small
-    a.psplit = rows_split((long long)grid.x * grid.y, a.P, 8);
+    a.psplit = rows_split((long long)grid.x * grid.y, a.P, 8, true);
     if (a.psplit > 1) {
       static bool attr = false;
       cudaError_t e = set_smem(stolt_fwd_rows<LOGN, SHIFT, MINB, HALF, true>, smem_cap<LOGN>(true),

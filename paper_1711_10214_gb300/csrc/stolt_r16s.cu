@@ -31,7 +31,7 @@ namespace {
 // panel's tap words at once, needs about 128.
 template <int LOGN>
 constexpr int r16s_minb_adj() {
-  return LOGN == 10 ? 10 : (LOGN == 11 ? 5 : 2);
+  return LOGN == 10 ? 10 : (LOGN == 11 ? 5 : 3);
 }
 template <int LOGN>
 constexpr int r16s_minb_fwd() {
@@ -237,7 +237,7 @@ template <int LOGN, bool SHIFT, bool HALF>
 cudaError_t launch_fwd16s_h(const RowArgs& a0, cudaStream_t s) {
   constexpr int N = 1 << LOGN;
   RowArgs a = a0;
-  a.psplit = rows_split((long long)a.batch * a.Lh, a.P, r16s_minb_fwd<LOGN>());
+  a.psplit = rows_split((long long)a.batch * a.Lh, a.P, r16s_minb_fwd<LOGN>(), true);
   const size_t smem = (size_t)(N + a.ld) * sizeof(float2), cap = (size_t)2 * N * sizeof(float2);
   if (a.psplit > 1) {
     static bool attr = false;
@@ -266,15 +266,20 @@ cudaError_t launch_adj16s_h(const RowArgs& a, cudaStream_t s) {
   const size_t smem = (size_t)2 * N * sizeof(float2);
   cudaError_t e = set_smem(stolt_adj_rows16s<LOGN, SHIFT, HALF>, smem, attr);
   if (e != cudaSuccess) return e;
-  const int n = rows_split((long long)a.batch * a.Lh, a.P, r16s_minb_adj<LOGN>());
+  const int n = rows_split((long long)a.batch * a.Lh, a.P, r16s_minb_adj<LOGN>(), false);
   stolt_adj_rows16s<LOGN, SHIFT, HALF><<<dim3(a.batch, a.Lh, n), N / 16, smem, s>>>(a);
   return cudaGetLastError();
 }
 
+// At Nt 4096 the last pass is a radix-16 one, whose pruned form is slower than
+// the whole (5 gathers 1500 x 417, 24 panels: 732 against 659 us; capped at 80
+// registers for a third CTA 685).
 template <int LOGN, bool SHIFT>
 cudaError_t launch_adj16s(const RowArgs& a, cudaStream_t s) {
-  return 2 * a.nt <= a.Nt ? launch_adj16s_h<LOGN, SHIFT, true>(a, s)
-                          : launch_adj16s_h<LOGN, SHIFT, false>(a, s);
+  if constexpr (LOGN < 12) {
+    if (2 * a.nt <= a.Nt) return launch_adj16s_h<LOGN, SHIFT, true>(a, s);
+  }
+  return launch_adj16s_h<LOGN, SHIFT, false>(a, s);
 }
 
 }  // namespace
