@@ -95,6 +95,9 @@ struct RowArgs {
 
 cudaError_t launch_xfft_r2c(const XfftArgs& a, cudaStream_t s);
 cudaError_t launch_xfft_c2r(const XfftArgs& a, cudaStream_t s);
+// Forms for panels that fill at most half of the padded axis (xfft_half.cu).
+bool xfft_half_applies(const XfftArgs& a);
+cudaError_t launch_xfft_r2c_half(const XfftArgs& a, cudaStream_t s);
 cudaError_t launch_stolt_fwd_rows(const RowArgs& a, cudaStream_t s);
 cudaError_t launch_stolt_adj_rows(const RowArgs& a, cudaStream_t s);
 // Radix-16 row kernels (Nt = 1024, 2048, 4096 only; see stolt_r16.cu).

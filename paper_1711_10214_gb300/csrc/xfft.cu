@@ -24,6 +24,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "tma.cuh"
+#include "xfft_common.cuh"
 
 namespace ashrt {
 
@@ -64,81 +65,6 @@ __device__ __forceinline__ void col_pass_range(float2* sm, const float2* __restr
   }
 }
 
-__device__ __forceinline__ double warp_sum(double x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
-}
-
-// Adds the CTA-wide sum of `part` to *dst (one atomic per CTA).
-__device__ __forceinline__ void block_accumulate(double part, double* dst) {
-  __shared__ double red[32];
-  part = warp_sum(part);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0) red[w] = part;
-  __syncthreads();
-  if (w == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-    double x = lane < nw ? red[lane] : 0.0;
-    x = warp_sum(x);
-    if (lane == 0) atomicAdd(dst, x);
-  }
-}
-
-// Real time samples t and t+1 of one trace, packed as z = x_t + i x_{t+1}
-// (one 8-byte load when the row is 8-byte aligned).
-__device__ __forceinline__ float2 load_pair_real(const float* __restrict__ row, int t, int nt,
-                                                 bool vec) {
-  if (vec && t + 1 < nt) return __ldg((const float2*)(row + t));
-  return make_float2(t < nt ? __ldg(row + t) : 0.f, t + 1 < nt ? __ldg(row + t + 1) : 0.f);
-}
-
-// Plain (coherent) pair load / store of samples t, t+1 of a row, for the
-// in-place CGLS updates (each pair is read and written by one thread).
-__device__ __forceinline__ float2 ld_pair(const float* row, int t, int nt, bool vec) {
-  if (vec && t + 1 < nt) return *(const float2*)(row + t);
-  return make_float2(t < nt ? row[t] : 0.f, t + 1 < nt ? row[t + 1] : 0.f);
-}
-
-__device__ __forceinline__ void st_pair(float* row, int t, int nt, bool vec, float2 v) {
-  if (vec && t + 1 < nt) {
-    *(float2*)(row + t) = v;
-    return;
-  }
-  if (t < nt) row[t] = v.x;
-  if (t + 1 < nt) row[t + 1] = v.y;
-}
-
-// The fused CGLS update of one sample pair (see XfftArgs::cg_mode); returns
-// the updated vector's pair, which is what the transform consumes.
-__device__ __forceinline__ float2 cg_update_pair(const XfftArgs& a, long long off, int t, bool vec,
-                                                 float4 cf) {
-  float* io = a.cg_io + off;
-  const float2 x = ld_pair(io, t, a.nt, vec);
-  const float2 y = ld_pair(a.cg_s + off, t, a.nt, vec);
-  float2 z;
-  if (a.cg_mode == 1) {
-    float* po = a.cg_pout ? a.cg_pout + off : io;
-    z = make_float2(fmaf(cf.x, y.x, cf.y * x.x), fmaf(cf.x, y.y, cf.y * x.y));
-    const bool two = a.cg_p2_read && cf.w != 0.f;
-    if (a.cg_u_rw && (cf.z != 0.f || two)) {
-      float* u = a.cg_u + off;
-      float2 un = ld_pair(u, t, a.nt, vec);
-      if (two) {
-        const float2 p2 = ld_pair(po, t, a.nt, vec);   // read before z overwrites it
-        un = make_float2(fmaf(cf.w, p2.x, un.x), fmaf(cf.w, p2.y, un.y));
-      }
-      un = make_float2(fmaf(cf.z, x.x, un.x), fmaf(cf.z, x.y, un.y));
-      st_pair(u, t, a.nt, vec, un);
-    }
-    st_pair(po, t, a.nt, vec, z);
-  } else {
-    z = make_float2(fmaf(-cf.z, y.x, x.x), fmaf(-cf.z, y.y, x.y));
-    st_pair(io, t, a.nt, vec, z);
-  }
-  return z;
-}
-
 template <int LOGN, int C>
 __global__ void __launch_bounds__((1 << LOGN) * C / 16)
 xfft_r2c_kernel(XfftArgs a) {
@@ -146,8 +72,9 @@ xfft_r2c_kernel(XfftArgs a) {
   using S = Sched<LOGN>;
   extern __shared__ float2 sm[];   // [N][C]
   const int tid = threadIdx.x, col = tid % C, j0 = tid / C;
-  const long long slab = blockIdx.x;
-  const int t0 = blockIdx.y * 2 * C;
+  const TileAt at = tile_at(a.nt, 2 * C);
+  const long long slab = at.slab;
+  const int t0 = at.t0;
   const int ta = t0 + 2 * col;      // this thread packs columns ta (real) and ta + 1 (imag)
   const bool vec = (a.nt & 1) == 0;
   const float* in = a.in_real + slab * a.slab_real;
@@ -376,23 +303,6 @@ xfft_r2c_tma(XfftArgs a, const __grid_constant__ R2cMaps mp, int n_tt, long long
   if (tid == 0) bulk_wait_all();
 }
 
-// Stored row `row` (<= N/2) of the half spectrum for the two adjacent columns
-// t and t+1 (t even): (A, B) = (re, im of column t, re, im of column t+1).
-// Rows are ld >= nt long with ld a multiple of 4, so the 16-byte load at an
-// even t < nt stays inside the row; a column >= nt reads as zero.
-__device__ __forceinline__ float4 col_load2(const float2* __restrict__ base, int ld, int row, int t,
-                                            int nt) {
-  const bool ok = t < nt, okb = t + 1 < nt;
-  const float4 y = __ldg((const float4*)(base + (long long)row * ld + (ok ? t : 0)));
-  return make_float4(ok ? y.x : 0.f, ok ? y.y : 0.f, okb ? y.z : 0.f, okb ? y.w : 0.f);
-}
-// Z = A + i B of a stored row (zdir), of its mirror N - row, whose A and B
-// are the conjugates (zmir), and of rows 0 and N/2, whose imaginary parts a
-// real signal's spectrum does not have (zreal).
-__device__ __forceinline__ float2 zdir(float4 y) { return make_float2(y.x - y.w, y.y + y.z); }
-__device__ __forceinline__ float2 zmir(float4 y) { return make_float2(y.x + y.w, y.z - y.y); }
-__device__ __forceinline__ float2 zreal(float4 y) { return make_float2(y.x, y.z); }
-
 // PF: the tile of the elementwise weight ew that this CTA's outputs use
 // ([nx][2C] floats) is copied into shared memory with cp.async when the CTA
 // starts, so the epilogue reads it from there instead of waiting on global
@@ -407,8 +317,9 @@ xfft_c2r_kernel(XfftArgs a) {
   using S = Sched<LOGN>;
   extern __shared__ float2 sm[];   // [N][C], then (PF) the weight tile [nx][2C] floats
   const int tid = threadIdx.x, col = tid % C, j0 = tid / C;
-  const long long slab = blockIdx.x;
-  const int t0 = blockIdx.y * 2 * C;
+  const TileAt at = tile_at(a.nt, 2 * C);
+  const long long slab = at.slab;
+  const int t0 = at.t0;
   const int ta = t0 + 2 * col;
   const float2* in = a.in_cplx + slab * a.slab_cplx;
   float* sew = (float*)(sm + N * C);
@@ -540,7 +451,7 @@ cudaError_t launch_r2c_v(const XfftArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  dim3 grid(a.slabs, (a.nt + 2 * C - 1) / (2 * C));
+  const unsigned grid = tile_grid(a.slabs, a.nt, 2 * C);
   xfft_r2c_kernel<LOGN, C><<<grid, T, smem, s>>>(a);
   return cudaGetLastError();
 }
@@ -599,7 +510,7 @@ cudaError_t launch_c2r_k(const XfftArgs& a, cudaStream_t s, size_t smem) {
     if (e != cudaSuccess) return e;
     attr = smem;
   }
-  dim3 grid(a.slabs, (a.nt + 2 * C - 1) / (2 * C));
+  const unsigned grid = tile_grid(a.slabs, a.nt, 2 * C);
   xfft_c2r_kernel<LOGN, C, PF, NXH><<<grid, T, smem, s>>>(a);
   return cudaGetLastError();
 }
@@ -664,6 +575,7 @@ cudaError_t launch_xfft_r2c(const XfftArgs& a, cudaStream_t s) {
     }
     if (e != cudaSuccess || used) return e;
   }
+  if (xfft_half_applies(a)) return launch_xfft_r2c_half(a, s);
   switch (xfft_log2(a.Nx)) {
     case 4: return launch_r2c_t<4>(a, s);
     case 5: return launch_r2c_t<5>(a, s);
