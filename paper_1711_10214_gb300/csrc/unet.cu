@@ -26,14 +26,6 @@ namespace {
 
 using bf16 = __nv_bfloat16;
 
-constexpr int kPix = 128;   // pixels (along a row) per CTA
-constexpr int kCh = 16;     // input / output channel tile
-
-template <typename T>
-__device__ __forceinline__ float ld_f(const T* p, long long i);
-template <>
-__device__ __forceinline__ float ld_f<float>(const float* p, long long i) { return p[i]; }
-
 template <typename T>
 __device__ __forceinline__ void st_f(T* p, long long i, float v);
 template <>
@@ -41,198 +33,55 @@ __device__ __forceinline__ void st_f<float>(float* p, long long i, float v) { p[
 template <>
 __device__ __forceinline__ void st_f<bf16>(bf16* p, long long i, float v) { p[i] = __float2bfloat16(v); }
 
+// sum of w e^2 to about 2^-45 in FP32 pairs: exact products (fma residuals) and
+// Knuth's two-sum; the FP64 units are so few that three FP64 operations per
+// element bound the kernels that used them.
+struct SumSq2 {
+  float s = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(float w, float e) {
+    const float q = w * e, qe = fmaf(w, e, -q);
+    const float p = q * e, pe = fmaf(qe, e, fmaf(q, e, -p));
+    const float t = s + p, z = t - s;
+    c += ((s - (t - z)) + (p - z)) + pe;
+    s = t;
+  }
+  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+};
+
 struct Tensor {        // a channel slice of an NHWC buffer
   void* p = nullptr;
   int ps = 0;          // channels allocated per pixel
   int off = 0;         // first channel of the slice
 };
 
-struct ConvArgs {
-  Tensor in;           // input: fp32 gradients (the CUDA-core fallback of the backward)
-  Tensor mask;         // bf16 activation: multiply input by (mask > 0), or p == nullptr
-  const bf16* w;       // [K*K][Cin][Cout]
-  const float* bias;   // [Cout] or nullptr
-  Tensor out;
-  int N, H, W, Cin, Cout, relu;
-};
-
-// y[p, co] = bias[co] + sum_{tap, ci} x[p + tap, ci] * w[tap][ci][co], "same"
-// zero padding, optional ReLU.  CTA: 128 consecutive pixels of one image row
-// x 16 output channels; input channels in tiles of 16 staged in shared
-// memory (3 rows x 130 pixels with the halo) together with the weight tile.
-template <int K, typename TI, typename TO>
-__global__ void __launch_bounds__(kPix) k_conv(ConvArgs a) {
-  constexpr int R = K / 2, PW = kPix + 2 * R;
-  __shared__ float xs[K][kCh][PW + 1];
-  __shared__ __align__(16) float ws[K * K][kCh][kCh];
-  const int tid = threadIdx.x;
-  const int xt = (a.W + kPix - 1) / kPix;
-  const int row = blockIdx.x / xt;               // n * H + y
-  const int x0 = (blockIdx.x % xt) * kPix;
-  const int n = row / a.H, y = row % a.H;
-  const int co0 = blockIdx.y * kCh;
-  const TI* in = (const TI*)a.in.p;
-  const bf16* mk = (const bf16*)a.mask.p;
-  float acc[kCh];
-#pragma unroll
-  for (int c = 0; c < kCh; ++c) acc[c] = 0.f;
-
-  for (int ci0 = 0; ci0 < a.Cin; ci0 += kCh) {
-    for (int e = tid; e < K * PW * kCh; e += kPix) {
-      const int c = e % kCh, px = (e / kCh) % PW, r = e / (kCh * PW);
-      const int yy = y + r - R, xx = x0 + px - R, ci = ci0 + c;
-      float v = 0.f;
-      if (yy >= 0 && yy < a.H && xx >= 0 && xx < a.W && ci < a.Cin) {
-        const long long pix = ((long long)n * a.H + yy) * a.W + xx;
-        v = ld_f(in, pix * a.in.ps + a.in.off + ci);
-        if (mk && __bfloat162float(mk[pix * a.mask.ps + a.mask.off + ci]) <= 0.f) v = 0.f;
-      }
-      xs[r][c][px] = v;
-    }
-    for (int e = tid; e < K * K * kCh * kCh; e += kPix) {
-      const int co = e % kCh, ci = (e / kCh) % kCh, tap = e / (kCh * kCh);
-      float v = 0.f;
-      if (ci0 + ci < a.Cin && co0 + co < a.Cout)
-        v = __bfloat162float(a.w[((long long)tap * a.Cin + ci0 + ci) * a.Cout + co0 + co]);
-      ws[tap][ci][co] = v;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int ci = 0; ci < kCh; ++ci) {
-#pragma unroll
-      for (int tap = 0; tap < K * K; ++tap) {
-        const float v = xs[tap / K][ci][tid + tap % K];
-        const float4* wp = (const float4*)&ws[tap][ci][0];
-#pragma unroll
-        for (int q = 0; q < kCh / 4; ++q) {
-          const float4 w4 = wp[q];
-          acc[4 * q + 0] = fmaf(v, w4.x, acc[4 * q + 0]);
-          acc[4 * q + 1] = fmaf(v, w4.y, acc[4 * q + 1]);
-          acc[4 * q + 2] = fmaf(v, w4.z, acc[4 * q + 2]);
-          acc[4 * q + 3] = fmaf(v, w4.w, acc[4 * q + 3]);
-        }
-      }
-    }
-    __syncthreads();
-  }
-  const int xx = x0 + tid;
-  if (xx >= a.W) return;
-  const long long pix = ((long long)n * a.H + y) * a.W + xx;
-  TO* out = (TO*)a.out.p;
-#pragma unroll
-  for (int c = 0; c < kCh; ++c) {
-    const int co = co0 + c;
-    if (co >= a.Cout) break;
-    float v = acc[c] + (a.bias ? a.bias[co] : 0.f);
-    if (a.relu) v = fmaxf(v, 0.f);
-    st_f(out, pix * a.out.ps + a.out.off + co, v);
-  }
-}
-
-struct WgradArgs {
-  Tensor in;          // bf16 layer input
-  Tensor g;           // fp32 gradient of the layer output
-  Tensor mask;        // bf16 layer output (ReLU mask) or p == nullptr
-  float* gw;          // [Cout][Cin][K][K] fp32 (the master weights' layout), accumulated
-  float* gb;          // [Cout] fp32, accumulated
-  int N, H, W, Cin, Cout;
-  int rows_per;       // image rows (over all N*H) one CTA reduces before its atomics
-};
-
-// gw[co][ci][tap] += sum_p x[p + tap, ci] g_eff[p, co]; gb[co] += sum_p g_eff[p, co]
-// with g_eff = g (mask > 0).  CTA: a 128-pixel column strip of rows_per image
-// rows x 16 input x 16 output channels; thread (ci, co) accumulates all K*K
-// taps over the strip, then one atomic each.
-template <int K>
-__global__ void __launch_bounds__(256) k_wgrad(WgradArgs a) {
-  constexpr int R = K / 2, PW = kPix + 2 * R;
-  __shared__ float xs[K][kCh][PW + 1];
-  __shared__ float gs[kCh][kPix + 1];
-  const int tid = threadIdx.x;
-  const int xt = (a.W + kPix - 1) / kPix;
-  const int x0 = (blockIdx.x % xt) * kPix;
-  const int row0 = (blockIdx.x / xt) * a.rows_per;
-  const int row1 = min(row0 + a.rows_per, a.N * a.H);
-  const int ci0 = blockIdx.y * kCh, co0 = blockIdx.z * kCh;
-  const bf16* in = (const bf16*)a.in.p;
-  const float* g = (const float*)a.g.p;
-  const bf16* mk = (const bf16*)a.mask.p;
-  const int ci = tid / kCh, co = tid % kCh;
-  float acc[K * K];
-#pragma unroll
-  for (int t = 0; t < K * K; ++t) acc[t] = 0.f;
-  float gsum = 0.f;
-  for (int row = row0; row < row1; ++row) {
-    const int n = row / a.H, y = row % a.H;
-    for (int e = tid; e < K * PW * kCh; e += 256) {
-      const int c = e % kCh, px = (e / kCh) % PW, r = e / (kCh * PW);
-      const int yy = y + r - R, xx = x0 + px - R, cc = ci0 + c;
-      float v = 0.f;
-      if (yy >= 0 && yy < a.H && xx >= 0 && xx < a.W && cc < a.Cin)
-        v = __bfloat162float(in[(((long long)n * a.H + yy) * a.W + xx) * a.in.ps + a.in.off + cc]);
-      xs[r][c][px] = v;
-    }
-    for (int e = tid; e < kPix * kCh; e += 256) {
-      const int c = e % kCh, px = e / kCh;
-      const int xx = x0 + px, cc = co0 + c;
-      float v = 0.f;
-      if (xx < a.W && cc < a.Cout) {
-        const long long pix = ((long long)n * a.H + y) * a.W + xx;
-        v = g[pix * a.g.ps + a.g.off + cc];
-        if (mk && __bfloat162float(mk[pix * a.mask.ps + a.mask.off + cc]) <= 0.f) v = 0.f;
-      }
-      gs[c][px] = v;
-    }
-    __syncthreads();
-    for (int px = 0; px < kPix; ++px) {
-      const float gv = gs[co][px];
-      gsum += gv;
-#pragma unroll
-      for (int t = 0; t < K * K; ++t) acc[t] = fmaf(xs[t / K][ci][px + t % K], gv, acc[t]);
-    }
-    __syncthreads();
-  }
-  if (ci0 + ci < a.Cin && co0 + co < a.Cout) {
-#pragma unroll
-    for (int t = 0; t < K * K; ++t)
-      atomicAdd(&a.gw[((long long)(co0 + co) * a.Cin + ci0 + ci) * (K * K) + t], acc[t]);
-  }
-  if (ci == 0 && blockIdx.y == 0 && co0 + co < a.Cout) atomicAdd(&a.gb[co0 + co], gsum);
-}
-
-// 2x2 average pooling (forward, bf16) and its transpose (accumulated, fp32).
-__global__ void k_pool(Tensor in, Tensor out, int N, int H, int W, int C) {
-  const int Ho = H / 2, Wo = W / 2;
-  const long long total = (long long)N * Ho * Wo * C;
+// 2x2 average pooling (forward, bf16; 8 channels per thread, as k_up).
+__global__ void __launch_bounds__(256) k_pool(Tensor in, Tensor out, int N, int H, int W, int C) {
+  const int Ho = H / 2, Wo = W / 2, C8 = C / 8;
+  const long long total = (long long)N * Ho * Wo * C8;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C);
-    const long long p = i / C;
-    const int xo = (int)(p % Wo), yo = (int)((p / Wo) % Ho), n = (int)(p / ((long long)Wo * Ho));
-    float s = 0.f;
-    for (int dy = 0; dy < 2; ++dy)
-      for (int dx = 0; dx < 2; ++dx) {
-        const long long q = ((long long)n * H + 2 * yo + dy) * W + 2 * xo + dx;
-        s += __bfloat162float(((const bf16*)in.p)[q * in.ps + in.off + c]);
-      }
-    ((bf16*)out.p)[p * out.ps + out.off + c] = __float2bfloat16(0.25f * s);
-  }
-}
-
-__global__ void k_pool_bwd_acc(Tensor gout, Tensor gin, int N, int H, int W, int C) {
-  const long long total = (long long)N * H * W * C;   // H, W: full-resolution sizes
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C);
-    const long long p = i / C;
-    const int x = (int)(p % W), y = (int)((p / W) % H), n = (int)(p / ((long long)W * H));
-    const long long q = ((long long)n * (H / 2) + y / 2) * (W / 2) + x / 2;
-    ((float*)gin.p)[p * gin.ps + gin.off + c] += 0.25f * ((const float*)gout.p)[q * gout.ps + gout.off + c];
+    const int c = (int)(i % C8) * 8;
+    const long long p = i / C8;
+    const int xo = (int)(p % Wo);
+    const long long q = (2 * (p / Wo)) * W + 2 * xo;       // p / Wo = n Ho + yo, H even
+    const bf16* src = (const bf16*)in.p + in.off + c;
+    __align__(16) bf16 v[4][8], o[8];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      *(uint4*)v[k] = *(const uint4*)(src + (q + (k >> 1) * W + (k & 1)) * in.ps);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      float s = 0.f;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) s += __bfloat162float(v[k][j]);
+      o[j] = __float2bfloat16(0.25f * s);
+    }
+    *(uint4*)((bf16*)out.p + p * out.ps + out.off + c) = *(const uint4*)o;
   }
 }
 
 // nearest 2x upsampling (forward, bf16; 8 channels = 16 bytes per thread, C,
-// strides and offsets multiples of 8) and its transpose (fp32, written)
+// strides and offsets multiples of 8)
 __global__ void k_up(Tensor in, Tensor out, int N, int H, int W, int C) {   // H, W: output sizes
   const int C8 = C / 8;
   const long long total = (long long)N * H * W * C8;
@@ -250,23 +99,6 @@ __global__ void k_up(Tensor in, Tensor out, int N, int H, int W, int C) {   // H
   }
 }
 
-__global__ void k_up_bwd(Tensor gout, Tensor gin, int N, int H, int W, int C) {   // H, W: input (low-res) sizes
-  const long long total = (long long)N * H * W * C;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C);
-    const long long p = i / C;
-    const int x = (int)(p % W), y = (int)((p / W) % H), n = (int)(p / ((long long)W * H));
-    float s = 0.f;
-    for (int dy = 0; dy < 2; ++dy)
-      for (int dx = 0; dx < 2; ++dx) {
-        const long long q = ((long long)n * (2 * H) + 2 * y + dy) * (2 * W) + 2 * x + dx;
-        s += ((const float*)gout.p)[q * gout.ps + gout.off + c];
-      }
-    ((float*)gin.p)[p * gin.ps + gin.off + c] = s;
-  }
-}
-
 // gathers [N][nx][nt] -> bf16 image [N][nx][nt][1] scaled by 1/rms[n]
 __global__ void k_pack_in(const float* d, const float* rms, bf16* x, long long per, int N) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < per * N;
@@ -278,14 +110,12 @@ __global__ void k_pack_in(const float* d, const float* rms, bf16* x, long long p
 // atomic per CTA), then rms = sqrt(sum / per)
 __global__ void k_sumsq(const float* d, long long per, double* acc) {
   const int n = blockIdx.y;
-  double s = 0.0;
+  SumSq2 s;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < per;
-       i += (long long)gridDim.x * blockDim.x) {
-    const double v = d[n * per + i];
-    s += v * v;
-  }
+       i += (long long)gridDim.x * blockDim.x)
+    s.add(1.f, d[n * per + i]);
   __shared__ double red[256];
-  red[threadIdx.x] = s;
+  red[threadIdx.x] = s.value();
   __syncthreads();
   for (int o = blockDim.x / 2; o > 0; o >>= 1) {
     if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
@@ -299,103 +129,314 @@ __global__ void k_rms_fin(const double* acc, long long per, float* rms, int N) {
   if (n < N) rms[n] = (float)fmax(sqrt(acc[n] / (double)per), 1e-30);
 }
 
-// First layer (one input channel -> 16): one thread per pixel, the 3x3
-// neighbourhood from the BF16 image, weights [9][16] from shared memory,
-// 16 BF16 outputs written as two 16-byte vectors (out.ps, out.off multiples of 8).
-__global__ void k_conv_first(const bf16* x, const bf16* w, const float* bias, Tensor out, int N,
-                             int H, int W, int relu) {
-  __shared__ float ws[9][16];
+// First layer (one input channel -> 16): a thread takes four pixels of a row (W is
+// a multiple of 8), so that each weight read from shared memory serves four
+// products; the 3 x 6 neighbourhood comes from the BF16 image, 16 BF16 outputs per
+// pixel leave as two 16-byte vectors (out.ps, out.off multiples of 8).
+__global__ void __launch_bounds__(256) k_conv_first(const bf16* x, const bf16* w, const float* bias,
+                                                    Tensor out, int N, int H, int W, int relu) {
+  __shared__ __align__(16) float ws[9][16];
   __shared__ float bs[16];
   if (threadIdx.x < 144) ws[threadIdx.x / 16][threadIdx.x % 16] = __bfloat162float(w[threadIdx.x]);
   if (threadIdx.x < 16) bs[threadIdx.x] = bias[threadIdx.x];
   __syncthreads();
-  const long long total = (long long)N * H * W;
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < total;
-       p += (long long)gridDim.x * blockDim.x) {
-    const int xx = (int)(p % W);
-    const long long ny = p / W;
+  const int W4 = W / 4;
+  const long long total = (long long)N * H * W4;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const int x0 = (int)(i % W4) * 4;
+    const long long ny = i / W4;
     const int y = (int)(ny % H);
-    const long long n = ny / H;
-    float acc[16];
+    float v[3][6];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) acc[c] = bs[c];
+    for (int r = 0; r < 3; ++r) {
+      const bool ok = y + r >= 1 && y + r <= H;
+      const bf16* row = x + (ny + (ok ? r - 1 : 0)) * W + x0;
+      __align__(8) bf16 m[4];
+      *(uint2*)m = *(const uint2*)row;
+      v[r][0] = ok && x0 > 0 ? __bfloat162float(row[-1]) : 0.f;
+      v[r][5] = ok && x0 + 4 < W ? __bfloat162float(row[4]) : 0.f;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[r][1 + k] = ok ? __bfloat162float(m[k]) : 0.f;
+    }
+    float acc[4][16];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int c = 0; c < 16; ++c) acc[k][c] = bs[c];
 #pragma unroll
     for (int t = 0; t < 9; ++t) {
-      const int yy = y + t / 3 - 1, xc = xx + t % 3 - 1;
-      const float v = (yy >= 0 && yy < H && xc >= 0 && xc < W)
-                          ? __bfloat162float(x[(n * H + yy) * W + xc]) : 0.f;
 #pragma unroll
-      for (int c = 0; c < 16; ++c) acc[c] = fmaf(v, ws[t][c], acc[c]);
+      for (int q = 0; q < 4; ++q) {
+        const float4 w4 = *(const float4*)&ws[t][4 * q];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float e = v[t / 3][k + t % 3];
+          acc[k][4 * q] = fmaf(e, w4.x, acc[k][4 * q]);
+          acc[k][4 * q + 1] = fmaf(e, w4.y, acc[k][4 * q + 1]);
+          acc[k][4 * q + 2] = fmaf(e, w4.z, acc[k][4 * q + 2]);
+          acc[k][4 * q + 3] = fmaf(e, w4.w, acc[k][4 * q + 3]);
+        }
+      }
     }
-    __align__(16) bf16 o[16];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) o[c] = __float2bfloat16(relu ? fmaxf(acc[c], 0.f) : acc[c]);
-    bf16* dst = (bf16*)out.p + p * out.ps + out.off;
-    *(uint4*)dst = *(const uint4*)o;
-    *(uint4*)(dst + 8) = *(const uint4*)(o + 8);
+    for (int k = 0; k < 4; ++k) {
+      __align__(16) bf16 o[16];
+#pragma unroll
+      for (int c = 0; c < 16; ++c)
+        o[c] = __float2bfloat16(relu ? fmaxf(acc[k][c], 0.f) : acc[k][c]);
+      bf16* dst = (bf16*)out.p + (ny * W + x0 + k) * out.ps + out.off;
+      *(uint4*)dst = *(const uint4*)o;
+      *(uint4*)(dst + 8) = *(const uint4*)(o + 8);
+    }
   }
 }
 
-// The input of an input-gradient convolution on the tensor cores: the FP32
-// gradient of a layer's output, masked by the layer's ReLU (act > 0), rounded
-// to BF16 into a dense [pixels][C] buffer; 8 channels per thread (C, strides
-// and offsets multiples of 8).
-__global__ void k_gz_bf16(Tensor g, Tensor act, bf16* out, long long npix, int C) {
+// The inputs of the weight- and input-gradient kernels of a layer: the FP32
+// gradient of its output, masked by its ReLU (act > 0), rounded to BF16 into a
+// dense [pixels][C] buffer.  Where the gradient comes straight from another
+// layer's input-gradient convolution, that kernel's epilogue writes it; these two
+// form it from what arrives through an upsampling and through a skip connection
+// and a pooling.  Eight channels per thread (C, strides and offsets multiples
+// of 8).
+__device__ __forceinline__ void gz_store(const float* v, Tensor act, long long p, int c, bf16* out,
+                                         int C) {
+  __align__(16) bf16 m[8], o[8];
+  *(uint4*)m = *(const uint4*)((const bf16*)act.p + p * act.ps + act.off + c);
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    o[j] = __float2bfloat16(__bfloat162float(m[j]) <= 0.f ? 0.f : v[j]);
+  *(uint4*)(out + p * C + c) = *(const uint4*)o;
+}
+__device__ __forceinline__ void ld8(const Tensor& t, long long p, int c, float* v) {
+  const float4* q = (const float4*)((const float*)t.p + p * t.ps + t.off + c);
+  const float4 a = q[0], b = q[1];
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+  v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+
+// transpose of the nearest 2x upsampling (the sum of the four output pixels)
+__global__ void __launch_bounds__(256) k_up_bwd_gz(Tensor gout, Tensor act, bf16* out, int N, int H,
+                                                   int W, int C) {   // H, W: input (low-res) sizes
   const int C8 = C / 8;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < npix * C8;
+  const long long total = (long long)N * H * W * C8;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
-    const long long p = i / C8;
     const int c = (int)(i % C8) * 8;
-    const float4* gp = (const float4*)((const float*)g.p + p * g.ps + g.off + c);
-    const float4 g0 = gp[0], g1 = gp[1];
-    float v[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-    if (act.p) {
-      __align__(16) bf16 m[8];
-      *(uint4*)m = *(const uint4*)((const bf16*)act.p + p * act.ps + act.off + c);
+    const long long p = i / C8;
+    const int x = (int)(p % W);
+    const long long ny = p / W;
+    const long long q0 = (2 * ny) * (2 * W) + 2 * x;
+    float g[4][8], s[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (__bfloat162float(m[j]) <= 0.f) v[j] = 0.f;
-    }
-    __align__(16) bf16 o[8];
+    for (int k = 0; k < 4; ++k) ld8(gout, q0 + (k >> 1) * 2 * W + (k & 1), c, g[k]);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) o[j] = __float2bfloat16(v[j]);
-    *(uint4*)(out + p * C + c) = *(const uint4*)o;
+    for (int j = 0; j < 8; ++j) s[j] = ((g[0][j] + g[1][j]) + g[2][j]) + g[3][j];
+    gz_store(s, act, p, c, out, C);
   }
 }
 
-// NHWC head output [N][P][cout] -> planar [N][cout][P] (P = pixels): one
-// thread per pixel reads its C contiguous values; the planar stores of a warp
-// are contiguous
-__global__ void k_unpack_out(const float* y, float* out, long long P, int C, int N) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P * N;
+// gradient of a pooled skip connection: g plus a quarter of the pooled map's
+__global__ void __launch_bounds__(256) k_pool_bwd_gz(Tensor g, Tensor gpool, Tensor act, bf16* out,
+                                                     int N, int H, int W, int C) {
+  const int C8 = C / 8;
+  const long long total = (long long)N * H * W * C8;   // H, W: full-resolution sizes
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
-    const long long n = i / P, p = i % P;
-    for (int c = 0; c < C; ++c) out[(n * C + c) * P + p] = y[i * C + c];
+    const int c = (int)(i % C8) * 8;
+    const long long p = i / C8;
+    const int x = (int)(p % W);
+    const long long ny = p / W;                 // n * H + y, H even
+    float v[8], q[8];
+    ld8(g, p, c, v);
+    ld8(gpool, (ny / 2) * (W / 2) + x / 2, c, q);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = fmaf(0.25f, q[j], v[j]);
+    gz_store(v, act, p, c, out, C);
   }
 }
 
-// loss = sum_c lam_c mean_p (y - t)^2 with y NHWC [N][P][C], t planar [N][C][P]
-__global__ void k_mse(const float* y, const float* t, const float* lam, float* gy, long long P,
-                      int C, int N, double* loss) {
+// The head's backward in one pass over the outputs: with y, t planar [N][C][P]
+// (P pixels) and a = the head's BF16 input [N P][16],
+//   loss += sum_c lam_c mean (y - t)^2,   gy = its derivative (FP32, not stored),
+//   gz[p][:] = BF16 of the masked input gradient sum_c gy[p][c] w[c][:] (a > 0),
+//   gw[c][:] += sum_p gy[p][c] a[p][:],   gb[c] += sum_p gy[p][c],
+// all in FP32.  A CTA takes tiles of 128 pixels (one per thread) and, along the
+// grid's y, 32 output channels for gw; the y = 0 CTAs also form gz.  gy and the
+// tile's inputs meet in shared memory, where each warp adds its 32 pixels to its
+// own copy of gw: lane (ci, half) owns channels half, half + 2, ..  What bounds it
+// is HBM (y, t and the 16-channel maps once): 8 images 256 x 1024, 25 channels,
+// separate loss, weight- and input-gradient kernels 458 + 382 + 198 us and a mask
+// pass, this one see k_head_bwd's row in the launch list.
+constexpr int kHeadPix = 128, kHeadCh = 32;
+__global__ void __launch_bounds__(kHeadPix) k_head_bwd(const float* __restrict__ y,
+                                                       const float* __restrict__ t,
+                                                       const float* __restrict__ lam,
+                                                       const bf16* __restrict__ a,
+                                                       const bf16* __restrict__ w, bf16* gz,
+                                                       float* gw, float* gb, long long P, int C,
+                                                       int N, double* loss) {
+  constexpr int LD = kHeadPix + 4;
+  __shared__ __align__(16) float gys[kHeadCh][LD];
+  __shared__ __align__(16) float as[16][LD];
+  __shared__ double red[kHeadPix / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int cb = blockIdx.y * kHeadCh, ci = lane & 15, half = lane >> 4;
+  const bool first = blockIdx.y == 0;
   const double inv = 1.0 / ((double)P * N);
-  double s = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P * C * N;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C);
-    const long long p = (i / C) % P, n = i / (P * C);
-    const float l = lam ? lam[c] : 1.f;
-    const float e = y[i] - t[(n * C + c) * P + p];
-    s += (double)l * e * e;
-    gy[i] = (float)(2.0 * inv) * l * e;
-  }
-  __shared__ double red[256];
-  red[threadIdx.x] = s;
+  const float inv2 = (float)(2.0 * inv);
+  float acc[kHeadCh / 2], bacc = 0.f;
+#pragma unroll
+  for (int k = 0; k < kHeadCh / 2; ++k) acc[k] = 0.f;
+  for (int i = tid; i < kHeadCh * LD; i += kHeadPix) ((float*)gys)[i] = 0.f;   // channels >= C
   __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+  SumSq2 loss2;
+  const long long total = P * N;
+  for (long long t0 = blockIdx.x * (long long)kHeadPix; t0 < total;
+       t0 += (long long)gridDim.x * kHeadPix) {
+    const long long q = t0 + tid;
+    const bool ok = q < total;
+    const long long n = ok ? q / P : 0, p = ok ? q - n * P : 0;
+    float av[16], gd[16];
+    {
+      __align__(16) bf16 m[16];
+      *(uint4*)m = ok ? *(const uint4*)(a + q * 16) : make_uint4(0u, 0u, 0u, 0u);
+      *(uint4*)(m + 8) = ok ? *(const uint4*)(a + q * 16 + 8) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        av[j] = __bfloat162float(m[j]);
+        as[j][tid] = av[j];
+        gd[j] = 0.f;
+      }
+    }
+    const float* yp = y + n * C * P + p;
+    const float* tp = t + n * C * P + p;
+    const int c0 = first ? 0 : cb, c1 = first ? C : min(C, cb + kHeadCh);
+#pragma unroll 5
+    for (int c = c0; c < c1; ++c) {
+      const float l = __ldg(lam + c);
+      const float e = ok ? __ldg(yp + (long long)c * P) - __ldg(tp + (long long)c * P) : 0.f;
+      const float g = inv2 * l * e;
+      if (c >= cb && c < cb + kHeadCh) gys[c - cb][tid] = g;
+      if (first) {
+        loss2.add(l, e);
+        __align__(16) bf16 wv[16];
+        *(uint4*)wv = __ldg((const uint4*)(w + c * 16));
+        *(uint4*)(wv + 8) = __ldg((const uint4*)(w + c * 16 + 8));
+#pragma unroll
+        for (int j = 0; j < 16; ++j) gd[j] = fmaf(g, __bfloat162float(wv[j]), gd[j]);
+      }
+    }
+    if (first && ok) {
+      __align__(16) bf16 o[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) o[j] = __float2bfloat16(av[j] <= 0.f ? 0.f : gd[j]);
+      *(uint4*)(gz + q * 16) = *(const uint4*)o;
+      *(uint4*)(gz + q * 16 + 8) = *(const uint4*)(o + 8);
+    }
+    __syncwarp();
+    // the warp's own 32 pixels (its lanes wrote them)
+#pragma unroll 2
+    for (int px = warp * 32; px < warp * 32 + 32; px += 4) {
+      const float4 d = *(const float4*)&as[ci][px];
+#pragma unroll
+      for (int k = 0; k < kHeadCh / 2; ++k) {
+        const float4 g = *(const float4*)&gys[2 * k + half][px];
+        acc[k] = fmaf(g.x, d.x, fmaf(g.y, d.y, fmaf(g.z, d.z, fmaf(g.w, d.w, acc[k]))));
+      }
+    }
+#pragma unroll
+    for (int px = warp * 32; px < warp * 32 + 32; px += 4) {
+      const float4 g = *(const float4*)&gys[lane][px];
+      bacc += (g.x + g.y) + (g.z + g.w);
+    }
+    __syncwarp();
+  }
+  // the warps' sums, then one atomic per weight and CTA
+  __syncthreads();
+  float* sum = &gys[0][0];                       // [kHeadCh][17]
+  for (int v = 0; v < kHeadPix / 32; ++v) {
+    if (warp == v) {
+#pragma unroll
+      for (int k = 0; k < kHeadCh / 2; ++k) {
+        float* d = sum + (2 * k + half) * 17 + ci;
+        *d = v == 0 ? acc[k] : *d + acc[k];
+      }
+      float* d = sum + lane * 17 + 16;
+      *d = v == 0 ? bacc : *d + bacc;
+    }
     __syncthreads();
   }
-  if (threadIdx.x == 0) atomicAdd(loss, red[0] * inv);
+  for (int i = tid; i < kHeadCh * 17; i += kHeadPix) {
+    const int c = cb + i / 17, j = i % 17;
+    if (c < C) atomicAdd(j < 16 ? gw + c * 16 + j : gb + c, sum[i]);
+  }
+  if (!first) return;
+  double s = loss2.value();
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) red[warp] = s;
+  __syncthreads();
+  if (tid == 0) {
+    for (int i = 1; i < kHeadPix / 32; ++i) s += red[i];
+    atomicAdd(loss, s * inv);
+  }
+}
+
+// Weight and bias gradients of the first layer (one input channel, FP32): with
+// x the BF16 image and g the FP32 gradient of the layer's 16 outputs masked by
+// its ReLU, gw[co][tap] += sum_p g[p][co] x[p + tap].  Thread (pixel, half of the
+// channels) keeps 8 x 9 sums in registers; a CTA adds them over shared memory and
+// leaves one atomic per weight.  Bound by HBM (the gradient and the mask once).
+__global__ void __launch_bounds__(256) k_wgrad_first(const bf16* __restrict__ x, Tensor g, Tensor act,
+                                                     float* gw, float* gb, int N, int H, int W) {
+  __shared__ float red[8][2][80];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, h = tid & 1;
+  float acc[8][9], bs[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    bs[j] = 0.f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) acc[j][k] = 0.f;
+  }
+  const long long total = (long long)N * H * W;
+  for (long long p = blockIdx.x * 128LL + (tid >> 1); p < total; p += gridDim.x * 128LL) {
+    const int xx = (int)(p % W);
+    const long long ny = p / W;
+    const int yy = (int)(ny % H);
+    float v[8], xv[9];
+    ld8(g, p, 8 * h, v);
+    __align__(16) bf16 m[8];
+    *(uint4*)m = *(const uint4*)((const bf16*)act.p + p * act.ps + act.off + 8 * h);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const int y1 = yy + k / 3 - 1, x1 = xx + k % 3 - 1;
+      xv[k] = (y1 >= 0 && y1 < H && x1 >= 0 && x1 < W)
+                  ? __bfloat162float(x[p + (long long)(k / 3 - 1) * W + (k % 3 - 1)]) : 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const float gj = __bfloat162float(m[j]) <= 0.f ? 0.f : v[j];
+      bs[j] += gj;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) acc[j][k] = fmaf(xv[k], gj, acc[j][k]);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+      float r = k < 9 ? acc[j][k] : bs[j];
+      for (int o = 16; o > 1; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+      if (lane < 2) red[warp][lane][j * 10 + k] = r;
+    }
+  }
+  __syncthreads();
+  if (tid < 160) {
+    const int hh = tid / 80, e = tid % 80, co = 8 * hh + e / 10, k = e % 10;
+    float r = 0.f;
+    for (int w = 0; w < 8; ++w) r += red[w][hh][e];
+    atomicAdd(k < 9 ? gw + co * 9 + k : gb + co, r);
+  }
 }
 
 // Adam on the flat FP32 master parameters
@@ -544,18 +585,6 @@ __global__ void __launch_bounds__(256, 2) k_conv_mma(MmaConvArgs a) {
   }
 }
 
-// Outputs back in input units: model panels (channels < C-1) scale with the
-// data, residual weights max(|r|, eps)^((p-2)/2) with its power, so the last
-// channel (log W_r in normalised units) becomes exp(y) * rms^wr_pow.
-__global__ void k_rescale_out(float* y, const float* rms, long long P, int C, int N, float wr_pow) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P * C * N;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)((i / P) % C);
-    const float r = rms[i / (P * C)];
-    y[i] = (c < C - 1) ? y[i] * r : expf(y[i]) * powf(r, wr_pow);
-  }
-}
-
 // Training targets in normalised units from a solve's model m [N][C-1][P] and
 // final residual weights wr [N][P]: t = m / rms, log(wr) - wr_pow log(rms).
 __global__ void k_targets(const float* m, const float* wr, const float* rms, float* t,
@@ -568,21 +597,6 @@ __global__ void k_targets(const float* m, const float* wr, const float* rms, flo
     const float r = rms[n];
     t[i] = (c < C - 1) ? m[(n * (C - 1) + c) * P + p] / r
                        : logf(fmaxf(wr[n * P + p], 1e-30f)) - wr_pow * logf(r);
-  }
-}
-
-// The warm start in input units: m0 [N][C-1][P] and wr0 [N][P] from the
-// planar head output [N][C][P].
-__global__ void k_predict_out(const float* y, const float* rms, float* m0, float* wr0,
-                              long long P, int C, int N, float wr_pow) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P * N;
-       i += (long long)gridDim.x * blockDim.x) {
-    const long long n = i / P, p = i % P;
-    const float r = rms[n];
-    const float* yn = y + n * C * P + p;
-    if (m0)
-      for (int c = 0; c < C - 1; ++c) m0[(n * (C - 1) + c) * P + p] = yn[(long long)c * P] * r;
-    if (wr0) wr0[n * P + p] = expf(yn[(long long)(C - 1) * P]) * powf(r, wr_pow);
   }
 }
 
@@ -613,11 +627,10 @@ struct ashrt_unet {
   std::vector<void*> allocs;
   bf16 *x, *e1a, *cat1, *p1, *e2a, *cat2, *p2, *e3a, *cat3, *p3, *ba, *bb, *d3a, *d3b, *d2a, *d2b,
       *d1a, *d1b;
-  float *y, *gy, *g1a, *gcat1, *gp1, *g2a, *gcat2, *gp2, *g3a, *gcat3, *gp3, *gba, *gbb, *gd3a,
-      *gd3b, *gd2a, *gd2b, *gd1a, *gd1b;
+  float *y, *ynhwc = nullptr, *g1a, *gcat1, *gp1, *gcat2, *gp2, *gcat3, *gp3;
   float *rms, *lam;
   double* rmsacc;
-  bf16* gzb;   // BF16 masked output gradient of the layer being differentiated
+  bf16 *gza, *gzb;   // BF16 masked output gradients of two successive layers
   int* err;    // set by a tensor-core kernel whose bounded wait ran out
   double* loss;
   std::vector<float> lam_h;
@@ -638,26 +651,6 @@ Tensor T_(void* p, int ps, int off = 0) {
   t.ps = ps;
   t.off = off;
   return t;
-}
-
-template <int K, typename TI, typename TO>
-void conv(Tensor in, Tensor mask, const bf16* w, const float* bias, Tensor out, int N, int H,
-          int W, int Cin, int Cout, int relu, cudaStream_t s) {
-  ConvArgs a;
-  a.in = in;
-  a.mask = mask;
-  a.w = w;
-  a.bias = bias;
-  a.out = out;
-  a.N = N;
-  a.H = H;
-  a.W = W;
-  a.Cin = Cin;
-  a.Cout = Cout;
-  a.relu = relu;
-  dim3 grid((unsigned)((long long)N * H * ((W + kPix - 1) / kPix)), (Cout + kCh - 1) / kCh);
-  k_conv<K, TI, TO><<<grid, kPix, 0, s>>>(a);
-  count_launches(1);
 }
 
 // ---------------------------------------------------------------------------
@@ -702,6 +695,31 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity) {
   return false;
 }
 
+// Where a planar head output goes.  Channel c < C - 1 of image n: main + n
+// main_n + c P; the last one: last + n last_n (either may be null).  With rms the
+// outputs are returned in input units: the panels times rms[n], the last channel
+// as exp(y) rms[n]^wr_pow.
+struct HeadOut {
+  float *main = nullptr, *last = nullptr;
+  long long main_n = 0, last_n = 0;
+  const float* rms = nullptr;
+  float wr_pow = 0.f;
+};
+
+// Pixel-major head output [N][P][C] to its planar place: one thread per pixel.
+__global__ void k_unpack_out(const float* y, HeadOut h, long long P, int C, int N) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P * N;
+       i += (long long)gridDim.x * blockDim.x) {
+    const long long n = i / P, p = i % P;
+    const float r = h.rms ? h.rms[n] : 1.f;
+    const float* yi = y + i * C;
+    if (h.main)
+      for (int c = 0; c < C - 1; ++c) h.main[n * h.main_n + c * P + p] = h.rms ? yi[c] * r : yi[c];
+    if (h.last)
+      h.last[n * h.last_n + p] = h.rms ? expf(yi[C - 1]) * powf(r, h.wr_pow) : yi[C - 1];
+  }
+}
+
 struct TcConvArgs {
   Tensor in;             // bf16 NHWC slice, ps and off multiples of 8
   const bf16* w;         // [K*K][Cout][Cin]
@@ -709,7 +727,9 @@ struct TcConvArgs {
   Tensor out;            // bf16 or fp32 NHWC slice
   int N, H, W, Cin, Cout, relu;
   int* err;              // set to 1 if the MMA completion wait ran out
-  int planar = 0;        // 1: out.p is planar [N][Cout][H*W] (ps, off unused)
+  int planar = 0;        // 1: planar FP32 output as in `head` (out unused)
+  Tensor mask;           // BF16 activation: outputs where it is <= 0 are zeroed, or p == nullptr
+  HeadOut head;          // planar: where the outputs go
 };
 
 __device__ __forceinline__ void cp16(void* dst, const void* src, bool valid) {
@@ -757,25 +777,38 @@ __global__ void __launch_bounds__(256) k_conv_tc(TcConvArgs a) {
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = *tslot;
 
-  // asynchronous copies of channel chunk c into stage st (zero-filled outside the image)
+  // asynchronous copies of channel chunk c into stage st (zero-filled outside the
+  // image): two threads per pixel, one 16-byte octet each, row by row; the 2 R
+  // halo pixels at the row's end by the first threads.  What a thread copies is
+  // the same in every chunk but for the channel, so its addresses are formed once.
+  const int sp = tid >> 1, so = tid & 1;
+  const bool okx = x0 + sp - R >= 0 && x0 + sp - R < a.W;
+  const long long rstride = (long long)a.W * a.in.ps;
+  const bf16* src0 = in + (((long long)n * a.H + y0 - R) * a.W + x0 + sp - R) * a.in.ps +
+                     a.in.off + 8 * so;
+  const int hr = tid >> 2, hp = 128 + (sp & 1);            // halo row and pixel
+  const bool okh = R > 0 && tid < 4 * ROWS && x0 + hp - R < a.W && y0 + hr - R >= 0 &&
+                   y0 + hr - R < a.H;
+  const bf16* srch = src0 + (long long)hr * rstride + (long long)(hp - sp) * a.in.ps;
   auto stage = [&](int c, int st) {
     unsigned char* As = smt + st * (A_BYTES + B_BYTES);
     unsigned char* Bs = As + A_BYTES;
     const int ci0 = c * 16;
-    for (int e = tid; e < ROWS * PW * 2; e += T) {
-      const int o = e % 2, px = (e / 2) % PW, r = e / (2 * PW);
-      const int yy = y0 + r - R, xx = x0 + px - R;
-      const bool ok = yy >= 0 && yy < a.H && xx >= 0 && xx < a.W;
-      const bf16* src = ok ? in + (((long long)n * a.H + yy) * a.W + xx) * a.in.ps + a.in.off +
-                                 ci0 + 8 * o
-                           : in;
-      cp16(As + (r * 2 + o) * A_PLANE + px * 16, src, ok);
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+      const bool ok = okx && y0 + r - R >= 0 && y0 + r - R < a.H;
+      cp16(As + (r * 2 + so) * A_PLANE + sp * 16, ok ? src0 + r * rstride + ci0 : in, ok);
     }
-    for (int e = tid; e < TAPS * NT * 2; e += T) {
-      const int o = e % 2, c = (e / 2) % NT, tap = e / (2 * NT);
-      const bool ok = co0 + c < a.Cout;
-      const bf16* src = ok ? a.w + ((long long)tap * a.Cout + co0 + c) * a.Cin + ci0 + 8 * o : a.w;
-      cp16(Bs + (tap * 2 + o) * B_PLANE + c * 16, src, ok);
+    if (R > 0 && tid < 4 * ROWS)
+      cp16(As + (hr * 2 + so) * A_PLANE + hp * 16, okh ? srch + ci0 : in, okh);
+#pragma unroll
+    for (int i = 0; i < (TAPS * NT + 127) / 128; ++i) {
+      const int e = sp + 128 * i, c = e % NT, tap = e / NT;
+      if (e < TAPS * NT) {
+        const bool ok = co0 + c < a.Cout;
+        const bf16* src = ok ? a.w + ((long long)tap * a.Cout + co0 + c) * a.Cin + ci0 + 8 * so : a.w;
+        cp16(Bs + (tap * 2 + so) * B_PLANE + c * 16, src, ok);
+      }
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
@@ -868,13 +901,30 @@ __global__ void __launch_bounds__(256) k_conv_tc(TcConvArgs a) {
         }
         const bool whole = cb + 16 <= a.Cout;
         if (a.planar) {
-          // planar output [N][Cout][H*W]: the stores of a warp are contiguous
+          // the stores of a warp are contiguous
           const long long P = (long long)a.H * a.W, p = (long long)y * a.W + xx;
+          const float rms = a.head.rms ? a.head.rms[n] : 1.f;
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (cb + j < a.Cout) st_f(out, ((long long)n * a.Cout + cb + j) * P + p, f[j]);
+          for (int j = 0; j < 16; ++j) {
+            if (cb + j < a.Cout - 1) {
+              if (a.head.main)
+                a.head.main[n * a.head.main_n + (cb + j) * P + p] = a.head.rms ? f[j] * rms : f[j];
+            } else if (cb + j == a.Cout - 1 && a.head.last) {
+              a.head.last[n * a.head.last_n + p] =
+                  a.head.rms ? expf(f[j]) * powf(rms, a.head.wr_pow) : f[j];
+            }
+          }
         } else if (sizeof(TO) == 2 && whole && ((a.out.ps | a.out.off) & 7) == 0) {
           __align__(16) bf16 o[16];
+          if (a.mask.p) {
+            const uint4* mp = (const uint4*)((const bf16*)a.mask.p + pix * a.mask.ps + a.mask.off + cb);
+            __align__(16) bf16 m[16];
+            *(uint4*)m = mp[0];
+            *(uint4*)(m + 8) = mp[1];
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              if (__bfloat162float(m[j]) <= 0.f) f[j] = 0.f;
+          }
 #pragma unroll
           for (int j = 0; j < 16; ++j) o[j] = __float2bfloat16(f[j]);
           bf16* dst = (bf16*)out + pix * a.out.ps + a.out.off + cb;
@@ -930,10 +980,13 @@ void conv_tc_v(const TcConvArgs& a, cudaStream_t s) {
 // the mma.sync kernel)
 template <int K, typename TO>
 bool conv_tc(Tensor in, const bf16* w, const float* bias, Tensor out, int N, int H, int W,
-             int Cin, int Cout, int relu, int* err, cudaStream_t s, int planar = 0) {
+             int Cin, int Cout, int relu, int* err, cudaStream_t s, int planar = 0,
+             Tensor mask = Tensor(), HeadOut head = HeadOut()) {
   if (Cin % 16 != 0 || in.ps % 8 != 0 || in.off % 8 != 0) return false;
   TcConvArgs a;
   a.planar = planar;
+  a.mask = mask;
+  a.head = head;
   a.in = in;
   a.w = w;
   a.bias = bias;
@@ -1020,34 +1073,6 @@ void conv_mma(Tensor in, const bf16* w, const float* bias, Tensor out, int N, in
   }
 }
 
-template <int K>
-void wgrad(Tensor in, Tensor g, Tensor mask, float* gw, float* gb, int N, int H, int W, int Cin,
-           int Cout, cudaStream_t s) {
-  WgradArgs a;
-  a.in = in;
-  a.g = g;
-  a.mask = mask;
-  a.gw = gw;
-  a.gb = gb;
-  a.N = N;
-  a.H = H;
-  a.W = W;
-  a.Cin = Cin;
-  a.Cout = Cout;
-  const int xt = (W + kPix - 1) / kPix;
-  const long long ch_tiles = (long long)((Cin + kCh - 1) / kCh) * ((Cout + kCh - 1) / kCh);
-  const long long want_strips = (152LL * 8 + ch_tiles - 1) / ch_tiles;   // ~8 CTAs per SM
-  const long long rows = (long long)N * H;
-  long long strips_per_col = (want_strips + xt - 1) / xt;
-  if (strips_per_col > rows) strips_per_col = rows;
-  if (strips_per_col < 1) strips_per_col = 1;
-  a.rows_per = (int)((rows + strips_per_col - 1) / strips_per_col);
-  const long long nstrip = (rows + a.rows_per - 1) / a.rows_per;
-  dim3 grid((unsigned)(nstrip * xt), (Cin + kCh - 1) / kCh, (Cout + kCh - 1) / kCh);
-  k_wgrad<K><<<grid, 256, 0, s>>>(a);
-  count_launches(1);
-}
-
 // rms[g] of the n input gathers x [n][per]
 void compute_rms(ashrt_unet* u, const float* x, long long per, int n, cudaStream_t s) {
   cudaMemsetAsync(u->rmsacc, 0, sizeof(double) * n, s);
@@ -1056,26 +1081,35 @@ void compute_rms(ashrt_unet* u, const float* x, long long per, int n, cudaStream
   count_launches(2);
 }
 
-// Forward pass on `n` images already packed in u->x; writes u->y (NHWC fp32).
-// head_planar: write the head's output there as planar [n][cout][H*W]
-// (inference) instead of NHWC into u->y (training).
-void net_forward(ashrt_unet* u, int n, cudaStream_t s, float* head_planar = nullptr) {
+// Planar outputs [n][cout][P] at y.
+HeadOut head_planar(const ashrt_unet* u, float* y) {
+  HeadOut h;
+  const long long P = (long long)u->H * u->W;
+  h.main = y;
+  h.last = y + (u->cout - 1) * P;
+  h.main_n = h.last_n = u->cout * P;
+  return h;
+}
+
+// Forward pass on `n` images already packed in u->x; the head's output goes where
+// `head` says.
+void net_forward(ashrt_unet* u, int n, cudaStream_t s, const HeadOut& head) {
   const int H = u->H, W = u->W, c0 = u->ch[0], c1 = u->ch[1], c2 = u->ch[2], c3 = u->ch[3];
   const Tensor none = T_(nullptr, 0);
   auto& L = u->L;
   auto B = [&](int i) { return u->w + L[i].b_off; };
   auto grid = [&](long long cnt) { return grid1d(cnt); };
   // encoder
-  k_conv_first<<<grid((long long)n * H * W), 256, 0, s>>>(u->x, L[0].wf, B(0), T_(u->e1a, c0), n,
+  k_conv_first<<<grid((long long)n * H * W / 4), 256, 0, s>>>(u->x, L[0].wf, B(0), T_(u->e1a, c0), n,
                                                           H, W, 1);
   conv_mma<3, bf16>(T_(u->e1a, c0), L[1].wn, B(1), T_(u->cat1, c1 + c0, c1), n, H, W, c0, c0, 1, s, u->err);
-  k_pool<<<grid((long long)n * H * W / 4 * c0), 256, 0, s>>>(T_(u->cat1, c1 + c0, c1), T_(u->p1, c0), n, H, W, c0);
+  k_pool<<<grid((long long)n * H * W / 4 * c0 / 8), 256, 0, s>>>(T_(u->cat1, c1 + c0, c1), T_(u->p1, c0), n, H, W, c0);
   conv_mma<3, bf16>(T_(u->p1, c0), L[2].wn, B(2), T_(u->e2a, c1), n, H / 2, W / 2, c0, c1, 1, s, u->err);
   conv_mma<3, bf16>(T_(u->e2a, c1), L[3].wn, B(3), T_(u->cat2, c2 + c1, c2), n, H / 2, W / 2, c1, c1, 1, s, u->err);
-  k_pool<<<grid((long long)n * H * W / 16 * c1), 256, 0, s>>>(T_(u->cat2, c2 + c1, c2), T_(u->p2, c1), n, H / 2, W / 2, c1);
+  k_pool<<<grid((long long)n * H * W / 16 * c1 / 8), 256, 0, s>>>(T_(u->cat2, c2 + c1, c2), T_(u->p2, c1), n, H / 2, W / 2, c1);
   conv_mma<3, bf16>(T_(u->p2, c1), L[4].wn, B(4), T_(u->e3a, c2), n, H / 4, W / 4, c1, c2, 1, s, u->err);
   conv_mma<3, bf16>(T_(u->e3a, c2), L[5].wn, B(5), T_(u->cat3, c3 + c2, c3), n, H / 4, W / 4, c2, c2, 1, s, u->err);
-  k_pool<<<grid((long long)n * H * W / 64 * c2), 256, 0, s>>>(T_(u->cat3, c3 + c2, c3), T_(u->p3, c2), n, H / 4, W / 4, c2);
+  k_pool<<<grid((long long)n * H * W / 64 * c2 / 8), 256, 0, s>>>(T_(u->cat3, c3 + c2, c3), T_(u->p3, c2), n, H / 4, W / 4, c2);
   conv_mma<3, bf16>(T_(u->p3, c2), L[6].wn, B(6), T_(u->ba, c3), n, H / 8, W / 8, c2, c3, 1, s, u->err);
   conv_mma<3, bf16>(T_(u->ba, c3), L[7].wn, B(7), T_(u->bb, c3), n, H / 8, W / 8, c3, c3, 1, s, u->err);
   // decoder
@@ -1088,15 +1122,14 @@ void net_forward(ashrt_unet* u, int n, cudaStream_t s, float* head_planar = null
   k_up<<<grid((long long)n * H * W * c1 / 8), 256, 0, s>>>(T_(u->d2b, c1), T_(u->cat1, c1 + c0, 0), n, H, W, c1);
   conv_mma<3, bf16>(T_(u->cat1, c1 + c0), L[12].wn, B(12), T_(u->d1a, c0), n, H, W, c1 + c0, c0, 1, s, u->err);
   conv_mma<3, bf16>(T_(u->d1a, c0), L[13].wn, B(13), T_(u->d1b, c0), n, H, W, c0, c0, 1, s, u->err);
-  if (!head_planar || !conv_tc<1, float>(T_(u->d1b, c0), L[14].wn, B(14), T_(head_planar, 1), n, H,
-                                         W, c0, u->cout, 0, u->err, s, 1)) {
-    conv_mma<1, float>(T_(u->d1b, c0), L[14].wn, B(14), T_(u->y, u->cout), n, H, W, c0, u->cout,
+  if (!conv_tc<1, float>(T_(u->d1b, c0), L[14].wn, B(14), none, n, H, W, c0, u->cout, 0, u->err, s, 1,
+                         none, head)) {
+    // a head wider than the tcgen05 tiles: pixel-major, then to its planar place
+    const long long P = (long long)H * W;
+    conv_mma<1, float>(T_(u->d1b, c0), L[14].wn, B(14), T_(u->ynhwc, u->cout), n, H, W, c0, u->cout,
                        0, s);
-    if (head_planar) {
-      k_unpack_out<<<grid1d((long long)H * W * n), 256, 0, s>>>(u->y, head_planar,
-                                                               (long long)H * W, u->cout, n);
-      count_launches(1);
-    }
+    k_unpack_out<<<grid1d(P * n), 256, 0, s>>>(u->ynhwc, head, P, u->cout, n);
+    count_launches(1);
   }
   count_launches(7);   // pools, upsamplings, first layer
 }
@@ -1104,12 +1137,18 @@ void net_forward(ashrt_unet* u, int n, cudaStream_t s, float* head_planar = null
 // Weight and bias gradients of a 3x3 layer on the tensor cores (mma.sync
 // m16n8k16, BF16 operands, FP32 accumulation): for every tap, an implicit GEMM
 // gw[co][ci] += sum_p gz[p][co] x[p + tap][ci] over the pixels p, M = output
-// channels, N = input channels, K = pixels.  A CTA owns 16 MT output x 32 input
-// channels and all nine taps and reduces a 128-pixel column strip of rows_per
-// image rows: per row it stages the BF16 masked output gradient [128][16 MT]
-// and the three input rows [3][130][32] in their NHWC order and reads both
-// operands with ldmatrix.trans; the FP32 partial sums leave with one atomic
-// each.  CTAs of the first input-channel tile also sum the bias gradient.
+// channels, N = input channels, K = pixels.  A CTA has nine warps, one per tap,
+// owns 16 MT output x 8 NT input channels and reduces a 128-pixel column strip of
+// rows_per image rows.  The input rows live in a ring of four: a row of output
+// gradients [128][16 MT] needs three of them, of which two are there already,
+// and the fourth is in flight with the next row of gradients, so every input row
+// is copied once and no copy is waited for.  Both operands stay in their NHWC
+// order and are read with ldmatrix.trans (row pitches of an odd number of 16-byte
+// units: no bank conflicts); a tap that looks across the image's first or last
+// row is left out for that row.  The FP32 partial sums leave with one atomic
+// each; CTAs of the first input-channel tile also sum the bias gradient.
+// Channel tiles of 48 x 48 (the network's channels are multiples of 48 but for
+// 16 and 64) waste nothing where 32 x 32 computed a third to a half of padding.
 struct WgMmaArgs {
   Tensor in;            // bf16 layer input slice (ps, off multiples of 8)
   const bf16* gz;       // bf16 masked output gradient, dense [pixels][Cout]
@@ -1125,190 +1164,213 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t& r0, uint32_t& r1, uint32_t& 
                : "r"((unsigned)__cvta_generic_to_shared(p)));
 }
 
-__device__ __forceinline__ void ldsm_x2_t(uint32_t& r0, uint32_t& r1, const void* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];\n"
-               : "=r"(r0), "=r"(r1)
-               : "r"((unsigned)__cvta_generic_to_shared(p)));
-}
-
-template <int MT>
-__global__ void __launch_bounds__(256) k_wgrad_mma(WgMmaArgs a) {
-  constexpr int CO_T = 16 * MT, CI_T = 32, LDX = CI_T + 8, LDG = CO_T + 8, PW = 130;
-  constexpr int TILES = 9 * MT * 4, PER = (TILES + 7) / 8;
-  __shared__ __align__(16) bf16 xs[3 * PW * LDX];
-  __shared__ __align__(16) bf16 gs[128 * LDG];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+template <int MT, int NT>
+__global__ void __launch_bounds__(288, MT * NT >= 18 ? 2 : 3) k_wgrad_mma(WgMmaArgs a) {
+  constexpr int CO_T = 16 * MT, CI_T = 8 * NT, LDX = CI_T + 8, LDG = CO_T + 8, PW = 130, T = 288;
+  constexpr int PARTS = T / CO_T;               // bias: threads per output channel
+  extern __shared__ __align__(16) unsigned char smw[];
+  bf16* xs = (bf16*)smw;                        // [4 rows][PW][LDX]
+  bf16* gs = xs + 4 * PW * LDX;                 // [2 rows][128][LDG]
+  const int tid = threadIdx.x, tap = tid >> 5, lane = tid & 31, dy = tap / 3, dx = tap % 3;
   const int xt = (a.W + 127) / 128;
   const int x0 = (blockIdx.x % xt) * 128;
-  const int row0 = (blockIdx.x / xt) * a.rows_per;
-  const int row1 = min(row0 + a.rows_per, a.N * a.H);
+  const int rows = a.N * a.H, row0 = (blockIdx.x / xt) * a.rows_per;
+  const int row1 = min(row0 + a.rows_per, rows);
   const int ci0 = blockIdx.y * CI_T, co0 = blockIdx.z * CO_T;
   const bf16* in = (const bf16*)a.in.p;
-  float acc[PER][4];
+  // input row R (over all images) into its place in the ring, and a row of output
+  // gradients: two threads per pixel with adjacent 16-byte octets (one 32-byte
+  // sector), the octets in steps of two
+  const int sp = tid >> 1, so = (tid & 1) * 8;
+  const bool okx = sp < PW && x0 + sp >= 1 && x0 + sp - 1 < a.W, okg = x0 + sp < a.W;
+  const bf16* srcx = in + (long long)(x0 + sp - 1) * a.in.ps + a.in.off + ci0 + so;
+  const bf16* srcg = a.gz + (long long)(x0 + sp) * a.Cout + co0 + so;
+  auto load_x = [&](int R) {
+    if (R < 0 || R >= rows || sp >= PW) return;   // (only taps that are left out would read R)
+    bf16* dst = xs + ((R & 3) * PW + sp) * LDX + so;
+    const bf16* src = srcx + (long long)R * a.W * a.in.ps;
 #pragma unroll
-  for (int j = 0; j < PER; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-  float bsum = 0.f;
-
-  for (int row = row0; row < row1; ++row) {
-    const int n = row / a.H, y = row % a.H;
-    for (int e = tid; e < 3 * PW * 4; e += 256) {
-      const int q = e % 4, px = (e / 4) % PW, r = e / (4 * PW);
-      const int yy = y + r - 1, xx = x0 + px - 1, c = ci0 + 8 * q;
-      const bool ok = yy >= 0 && yy < a.H && xx >= 0 && xx < a.W && c < a.Cin;
-      const bf16* src = ok ? in + (((long long)n * a.H + yy) * a.W + xx) * a.in.ps + a.in.off + c : in;
-      cp16(xs + (r * PW + px) * LDX + 8 * q, src, ok);
+    for (int q = 0; q < NT / 2; ++q) {
+      const bool ok = okx && ci0 + 16 * q < a.Cin;
+      cp16(dst + 16 * q, ok ? src + 16 * q : in, ok);
     }
-    for (int e = tid; e < 128 * (CO_T / 8); e += 256) {
-      const int q = e % (CO_T / 8), px = e / (CO_T / 8);
-      const int xx = x0 + px, c = co0 + 8 * q;
-      const bool ok = xx < a.W && c < a.Cout;
-      const bf16* src = ok ? a.gz + (((long long)n * a.H + y) * a.W + xx) * a.Cout + c : a.gz;
-      cp16(gs + px * LDG + 8 * q, src, ok);
+  };
+  auto load_g = [&](int R) {
+    if (sp >= 128) return;
+    bf16* dst = gs + ((R & 1) * 128 + sp) * LDG + so;
+    const bf16* src = srcg + (long long)R * a.W * a.Cout;
+#pragma unroll
+    for (int q = 0; q < MT; ++q) {
+      const bool ok = okg && co0 + 16 * q < a.Cout;
+      cp16(dst + 16 * q, ok ? src + 16 * q : a.gz, ok);
+    }
+  };
+  float acc[MT][NT][4];
+#pragma unroll
+  for (int i = 0; i < MT; ++i)
+#pragma unroll
+    for (int j = 0; j < NT; ++j) acc[i][j][0] = acc[i][j][1] = acc[i][j][2] = acc[i][j][3] = 0.f;
+  float bsum = 0.f;
+  const bool bias = blockIdx.y == 0 && tid < PARTS * CO_T;
+
+  load_x(row0 - 1);
+  load_x(row0);
+  load_x(row0 + 1);
+  load_g(row0);
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+  for (int row = row0; row < row1; ++row) {
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();   // this row's operands are there; the previous row's reads are done
+    if (row + 1 < row1) {
+      load_x(row + 2);
+      load_g(row + 1);
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    __syncthreads();
-    if (blockIdx.y == 0 && tid < CO_T)
-      for (int px = 0; px < 128; ++px) bsum += __bfloat162float(gs[px * LDG + tid]);
+    const bf16* g = gs + (row & 1) * 128 * LDG;
+    if (bias)
+      for (int px = tid / CO_T; px < 128; px += PARTS)
+        bsum += __bfloat162float(g[px * LDG + tid % CO_T]);
+    const int y = row % a.H;
+    if ((dy == 0 && y == 0) || (dy == 2 && y == a.H - 1)) continue;
+    const bf16* x = xs + ((row + dy - 1) & 3) * PW * LDX + dx * LDX;
+    const int kr = lane & 7, id = lane >> 3;
 #pragma unroll 2
     for (int kb = 0; kb < 128; kb += 16) {
       uint32_t af[MT][4];
 #pragma unroll
-      for (int mt = 0; mt < MT; ++mt) {
-        const int kr = kb + (lane & 7) + ((lane >> 4) << 3), mc = mt * 16 + (((lane >> 3) & 1) << 3);
-        ldsm_x4_t(af[mt][0], af[mt][1], af[mt][2], af[mt][3], gs + kr * LDG + mc);
-      }
+      for (int i = 0; i < MT; ++i)
+        ldsm_x4_t(af[i][0], af[i][1], af[i][2], af[i][3],
+                  g + (kb + kr + ((id >> 1) << 3)) * LDG + i * 16 + ((id & 1) << 3));
 #pragma unroll
-      for (int j = 0; j < PER; ++j) {
-        const int id = warp + 8 * j;
-        if (id < TILES) {
-          const int tap = id / (4 * MT), mt = (id / 4) % MT, nt = id % 4;
-          const int dy = tap / 3, dx = tap % 3;
-          const int kr = kb + dx + (lane & 7) + (((lane >> 3) & 1) << 3);
-          uint32_t b0, b1;
-          ldsm_x2_t(b0, b1, xs + (dy * PW + kr) * LDX + nt * 8);
-          // select the A fragment with conditionals (a register array indexed
-          // by a runtime value would live in local memory)
-          const bool m1 = MT > 1 && mt == 1;
-          mma_bf16(acc[j], m1 ? af[MT - 1][0] : af[0][0], m1 ? af[MT - 1][1] : af[0][1],
-                   m1 ? af[MT - 1][2] : af[0][2], m1 ? af[MT - 1][3] : af[0][3], b0, b1);
+      for (int j = 0; j < NT; j += 2) {
+        uint32_t b0, b1, b2, b3;
+        ldsm_x4_t(b0, b1, b2, b3, x + (kb + kr + ((id & 1) << 3)) * LDX + (j + (id >> 1)) * 8);
+#pragma unroll
+        for (int i = 0; i < MT; ++i) {
+          mma_bf16(acc[i][j], af[i][0], af[i][1], af[i][2], af[i][3], b0, b1);
+          mma_bf16(acc[i][j + 1], af[i][0], af[i][1], af[i][2], af[i][3], b2, b3);
         }
       }
     }
-    __syncthreads();
   }
   const int g = lane >> 2, t = lane & 3;
 #pragma unroll
-  for (int j = 0; j < PER; ++j) {
-    const int id = warp + 8 * j;
-    if (id >= TILES) continue;
-    const int tap = id / (4 * MT), mt = (id / 4) % MT, nt = id % 4;
+  for (int i = 0; i < MT; ++i)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int co = co0 + mt * 16 + g + 8 * h;
-      if (co >= a.Cout) continue;
+    for (int j = 0; j < NT; ++j)
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int ci = ci0 + nt * 8 + 2 * t + u;
-        if (ci < a.Cin) atomicAdd(&a.gw[((long long)co * a.Cin + ci) * 9 + tap], acc[j][2 * h + u]);
+      for (int e = 0; e < 4; ++e) {
+        const int co = co0 + i * 16 + g + 8 * (e >> 1), ci = ci0 + j * 8 + 2 * t + (e & 1);
+        if (co < a.Cout && ci < a.Cin)
+          atomicAdd(&a.gw[((long long)co * a.Cin + ci) * 9 + tap], acc[i][j][e]);
       }
-    }
-  }
-  if (blockIdx.y == 0 && tid < CO_T && co0 + tid < a.Cout) atomicAdd(&a.gb[co0 + tid], bsum);
+  if (bias && co0 + tid % CO_T < a.Cout) atomicAdd(&a.gb[co0 + tid % CO_T], bsum);
 }
 
-template <int MT>
+template <int MT, int NT>
 void wgrad_mma_v(const WgMmaArgs& a0, cudaStream_t s) {
   WgMmaArgs a = a0;
+  constexpr size_t smem = (size_t)(4 * 130 * (8 * NT + 8) + 2 * 128 * (16 * MT + 8)) * sizeof(bf16);
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(k_wgrad_mma<MT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    attr = true;
+  }
   const int xt = (a.W + 127) / 128;
-  const long long ch_tiles = (long long)((a.Cin + 31) / 32) * ((a.Cout + 16 * MT - 1) / (16 * MT));
-  const long long want = (152LL * 8 + ch_tiles - 1) / ch_tiles;
-  const long long rows = (long long)a.N * a.H;
-  long long per_col = (want + xt - 1) / xt;
-  per_col = std::max(1LL, std::min(per_col, rows));
+  const unsigned gy = (a.Cin + 8 * NT - 1) / (8 * NT), gz = (a.Cout + 16 * MT - 1) / (16 * MT);
+  // one wave of two or three CTAs per SM: each extra strip costs its atomics again
+  const int res = MT * NT >= 18 ? 2 : 3;
+  const long long rows = (long long)a.N * a.H, want = 152LL * res / ((long long)gy * gz * xt);
+  const long long per_col = std::max(1LL, std::min(want, rows));
   a.rows_per = (int)((rows + per_col - 1) / per_col);
   const long long nstrip = (rows + a.rows_per - 1) / a.rows_per;
-  dim3 grid((unsigned)(nstrip * xt), (a.Cin + 31) / 32, (a.Cout + 16 * MT - 1) / (16 * MT));
-  k_wgrad_mma<MT><<<grid, 256, 0, s>>>(a);
+  k_wgrad_mma<MT, NT><<<dim3((unsigned)(nstrip * xt), gy, gz), 288, smem, s>>>(a);
   count_launches(1);
 }
 
-// Backward of 3x3 layer l (input `in`, output gradient g masked by its ReLU
-// output act): weight and bias gradients and, if out.p, the input gradient.
-// On the tensor cores the masked gradient is rounded to BF16 once and serves
-// both products; otherwise the CUDA-core kernels work on the FP32 gradient.
-void layer_backward(ashrt_unet* u, Tensor in, Tensor g, Tensor act, const Layer& l, float* gw,
-                    float* gb, Tensor out, int n, int H, int W, int Cin, int Cout, cudaStream_t s) {
-  const long long npix = (long long)n * H * W;
-  const bool tc = Cin % 16 == 0 && Cout % 16 == 0 && ((in.ps | in.off) & 7) == 0 &&
-                  ((g.ps | g.off) & 7) == 0 && ((act.ps | act.off) & 7) == 0;
-  if (!tc) {
-    wgrad<3>(in, g, act, gw, gb, n, H, W, Cin, Cout, s);
-    if (out.p) conv<3, float, float>(g, act, l.wt, nullptr, out, n, H, W, Cout, Cin, 0, s);
-    return;
-  }
-  k_gz_bf16<<<grid1d(npix * Cout / 8), 256, 0, s>>>(g, act, u->gzb, npix, Cout);
-  count_launches(1);
+// Backward of 3x3 layer l (input `in`, BF16 masked output gradient gz): weight
+// and bias gradients, and the input gradient either as FP32 into `out` or, with
+// `act` (the ReLU output that is the layer's input), masked and rounded into
+// gz_out for the layer before.
+void layer_backward(ashrt_unet* u, Tensor in, const bf16* gz, const Layer& l, Tensor out,
+                    Tensor act, bf16* gz_out, int n, int H, int W, cudaStream_t s) {
   WgMmaArgs a;
   a.in = in;
-  a.gz = u->gzb;
-  a.gw = gw;
-  a.gb = gb;
+  a.gz = gz;
+  a.gw = u->g + l.w_off;
+  a.gb = u->g + l.b_off;
   a.N = n;
   a.H = H;
   a.W = W;
-  a.Cin = Cin;
-  a.Cout = Cout;
-  if (Cout <= 16) wgrad_mma_v<1>(a, s);
-  else wgrad_mma_v<2>(a, s);
-  if (out.p && !conv_tc<3, float>(T_(u->gzb, Cout), l.wtn, nullptr, out, n, H, W, Cout, Cin, 0,
-                                  u->err, s))
-    conv<3, float, float>(g, act, l.wt, nullptr, out, n, H, W, Cout, Cin, 0, s);
+  a.Cin = l.ci;
+  a.Cout = l.co;
+  // channel tiles 16 MT x 8 NT: the widest that divides both channel counts
+  if (l.co % 48 == 0) {
+    if (l.ci % 48 == 0) wgrad_mma_v<3, 6>(a, s);
+    else wgrad_mma_v<3, 2>(a, s);
+  } else {
+    if (l.ci % 32 == 0) wgrad_mma_v<1, 4>(a, s);
+    else wgrad_mma_v<1, 2>(a, s);
+  }
+  const Tensor g = T_(const_cast<bf16*>(gz), l.co);
+  if (gz_out)
+    conv_tc<3, bf16>(g, l.wtn, nullptr, T_(gz_out, l.ci), n, H, W, l.co, l.ci, 0, u->err, s, 0, act);
+  else
+    conv_tc<3, float>(g, l.wtn, nullptr, out, n, H, W, l.co, l.ci, 0, u->err, s);
 }
 
-// Backward pass from u->gy (NHWC fp32); accumulates parameter gradients in u->g.
-void net_backward(ashrt_unet* u, int n, cudaStream_t s) {
+// Backward pass from the planar head output u->y and the targets; accumulates
+// parameter gradients in u->g and the loss in u->loss.
+void net_backward(ashrt_unet* u, const float* target, int n, cudaStream_t s) {
   const int H = u->H, W = u->W, c0 = u->ch[0], c1 = u->ch[1], c2 = u->ch[2], c3 = u->ch[3];
   const Tensor none = T_(nullptr, 0);
   auto& L = u->L;
-  auto GW = [&](int i) { return u->g + L[i].w_off; };
-  auto GB = [&](int i) { return u->g + L[i].b_off; };
   auto grid = [&](long long cnt) { return grid1d(cnt); };
-  // Each conv layer i maps (input tensor in_i) -> (output act_i); given the
-  // gradient G of its output (masked by act_i > 0 when it has a ReLU):
-  //   wgrad(in_i, G, mask act_i) and, unless it is the first layer,
-  //   G_in = conv(G masked, flipped weights).
-  // head (no ReLU)
-  wgrad<1>(T_(u->d1b, c0), T_(u->gy, u->cout), none, GW(14), GB(14), n, H, W, c0, u->cout, s);
-  conv<1, float, float>(T_(u->gy, u->cout), none, L[14].wt, nullptr, T_(u->gd1b, c0), n, H, W, u->cout, c0, 0, s);
+  bf16 *ga = u->gza, *gb = u->gzb;   // masked output gradients of a layer and of the one before
+  const long long P = (long long)H * W;
+  const dim3 hg((unsigned)std::min<long long>((P * n + kHeadPix - 1) / kHeadPix, 152 * 8),
+                (u->cout + kHeadCh - 1) / kHeadCh);
+  k_head_bwd<<<hg, kHeadPix, 0, s>>>(u->y, target, u->lam, u->d1b, L[14].wt, ga,
+                                     u->g + L[14].w_off, u->g + L[14].b_off, P, u->cout, n, u->loss);
   // dec1
-  layer_backward(u, T_(u->d1a, c0), T_(u->gd1b, c0), T_(u->d1b, c0), L[13], GW(13), GB(13), T_(u->gd1a, c0), n, H, W, c0, c0, s);
-  layer_backward(u, T_(u->cat1, c1 + c0), T_(u->gd1a, c0), T_(u->d1a, c0), L[12], GW(12), GB(12), T_(u->gcat1, c1 + c0), n, H, W, c1 + c0, c0, s);
-  k_up_bwd<<<grid((long long)n * H * W / 4 * c1), 256, 0, s>>>(T_(u->gcat1, c1 + c0, 0), T_(u->gd2b, c1), n, H / 2, W / 2, c1);
+  layer_backward(u, T_(u->d1a, c0), ga, L[13], none, T_(u->d1a, c0), gb, n, H, W, s);
+  layer_backward(u, T_(u->cat1, c1 + c0), gb, L[12], T_(u->gcat1, c1 + c0), none, nullptr, n, H, W, s);
+  k_up_bwd_gz<<<grid(P * n / 4 * c1 / 8), 256, 0, s>>>(T_(u->gcat1, c1 + c0, 0), T_(u->d2b, c1), ga,
+                                                       n, H / 2, W / 2, c1);
   // dec2
-  layer_backward(u, T_(u->d2a, c1), T_(u->gd2b, c1), T_(u->d2b, c1), L[11], GW(11), GB(11), T_(u->gd2a, c1), n, H / 2, W / 2, c1, c1, s);
-  layer_backward(u, T_(u->cat2, c2 + c1), T_(u->gd2a, c1), T_(u->d2a, c1), L[10], GW(10), GB(10), T_(u->gcat2, c2 + c1), n, H / 2, W / 2, c2 + c1, c1, s);
-  k_up_bwd<<<grid((long long)n * H * W / 16 * c2), 256, 0, s>>>(T_(u->gcat2, c2 + c1, 0), T_(u->gd3b, c2), n, H / 4, W / 4, c2);
+  layer_backward(u, T_(u->d2a, c1), ga, L[11], none, T_(u->d2a, c1), gb, n, H / 2, W / 2, s);
+  layer_backward(u, T_(u->cat2, c2 + c1), gb, L[10], T_(u->gcat2, c2 + c1), none, nullptr, n, H / 2,
+                 W / 2, s);
+  k_up_bwd_gz<<<grid(P * n / 16 * c2 / 8), 256, 0, s>>>(T_(u->gcat2, c2 + c1, 0), T_(u->d3b, c2), ga,
+                                                        n, H / 4, W / 4, c2);
   // dec3
-  layer_backward(u, T_(u->d3a, c2), T_(u->gd3b, c2), T_(u->d3b, c2), L[9], GW(9), GB(9), T_(u->gd3a, c2), n, H / 4, W / 4, c2, c2, s);
-  layer_backward(u, T_(u->cat3, c3 + c2), T_(u->gd3a, c2), T_(u->d3a, c2), L[8], GW(8), GB(8), T_(u->gcat3, c3 + c2), n, H / 4, W / 4, c3 + c2, c2, s);
-  k_up_bwd<<<grid((long long)n * H * W / 64 * c3), 256, 0, s>>>(T_(u->gcat3, c3 + c2, 0), T_(u->gbb, c3), n, H / 8, W / 8, c3);
+  layer_backward(u, T_(u->d3a, c2), ga, L[9], none, T_(u->d3a, c2), gb, n, H / 4, W / 4, s);
+  layer_backward(u, T_(u->cat3, c3 + c2), gb, L[8], T_(u->gcat3, c3 + c2), none, nullptr, n, H / 4,
+                 W / 4, s);
+  k_up_bwd_gz<<<grid(P * n / 64 * c3 / 8), 256, 0, s>>>(T_(u->gcat3, c3 + c2, 0), T_(u->bb, c3), ga,
+                                                        n, H / 8, W / 8, c3);
   // bottleneck
-  layer_backward(u, T_(u->ba, c3), T_(u->gbb, c3), T_(u->bb, c3), L[7], GW(7), GB(7), T_(u->gba, c3), n, H / 8, W / 8, c3, c3, s);
-  layer_backward(u, T_(u->p3, c2), T_(u->gba, c3), T_(u->ba, c3), L[6], GW(6), GB(6), T_(u->gp3, c2), n, H / 8, W / 8, c2, c3, s);
-  k_pool_bwd_acc<<<grid((long long)n * H * W / 16 * c2), 256, 0, s>>>(T_(u->gp3, c2), T_(u->gcat3, c3 + c2, c3), n, H / 4, W / 4, c2);
+  layer_backward(u, T_(u->ba, c3), ga, L[7], none, T_(u->ba, c3), gb, n, H / 8, W / 8, s);
+  layer_backward(u, T_(u->p3, c2), gb, L[6], T_(u->gp3, c2), none, nullptr, n, H / 8, W / 8, s);
   // enc3 (its output s3 lives in cat3[c3:], gradient in gcat3[c3:])
-  layer_backward(u, T_(u->e3a, c2), T_(u->gcat3, c3 + c2, c3), T_(u->cat3, c3 + c2, c3), L[5], GW(5), GB(5), T_(u->g3a, c2), n, H / 4, W / 4, c2, c2, s);
-  layer_backward(u, T_(u->p2, c1), T_(u->g3a, c2), T_(u->e3a, c2), L[4], GW(4), GB(4), T_(u->gp2, c1), n, H / 4, W / 4, c1, c2, s);
-  k_pool_bwd_acc<<<grid((long long)n * H * W / 4 * c1), 256, 0, s>>>(T_(u->gp2, c1), T_(u->gcat2, c2 + c1, c2), n, H / 2, W / 2, c1);
+  k_pool_bwd_gz<<<grid(P * n / 16 * c2 / 8), 256, 0, s>>>(T_(u->gcat3, c3 + c2, c3), T_(u->gp3, c2),
+                                                          T_(u->cat3, c3 + c2, c3), ga, n, H / 4,
+                                                          W / 4, c2);
+  layer_backward(u, T_(u->e3a, c2), ga, L[5], none, T_(u->e3a, c2), gb, n, H / 4, W / 4, s);
+  layer_backward(u, T_(u->p2, c1), gb, L[4], T_(u->gp2, c1), none, nullptr, n, H / 4, W / 4, s);
   // enc2
-  layer_backward(u, T_(u->e2a, c1), T_(u->gcat2, c2 + c1, c2), T_(u->cat2, c2 + c1, c2), L[3], GW(3), GB(3), T_(u->g2a, c1), n, H / 2, W / 2, c1, c1, s);
-  layer_backward(u, T_(u->p1, c0), T_(u->g2a, c1), T_(u->e2a, c1), L[2], GW(2), GB(2), T_(u->gp1, c0), n, H / 2, W / 2, c0, c1, s);
-  k_pool_bwd_acc<<<grid((long long)n * H * W * c0), 256, 0, s>>>(T_(u->gp1, c0), T_(u->gcat1, c1 + c0, c1), n, H, W, c0);
-  // enc1
-  layer_backward(u, T_(u->e1a, c0), T_(u->gcat1, c1 + c0, c1), T_(u->cat1, c1 + c0, c1), L[1], GW(1), GB(1), T_(u->g1a, c0), n, H, W, c0, c0, s);
-  layer_backward(u, T_(u->x, 1), T_(u->g1a, c0), T_(u->e1a, c0), L[0], GW(0), GB(0), none, n, H, W, 1, c0, s);
-  count_launches(6);
+  k_pool_bwd_gz<<<grid(P * n / 4 * c1 / 8), 256, 0, s>>>(T_(u->gcat2, c2 + c1, c2), T_(u->gp2, c1),
+                                                         T_(u->cat2, c2 + c1, c2), ga, n, H / 2,
+                                                         W / 2, c1);
+  layer_backward(u, T_(u->e2a, c1), ga, L[3], none, T_(u->e2a, c1), gb, n, H / 2, W / 2, s);
+  layer_backward(u, T_(u->p1, c0), gb, L[2], T_(u->gp1, c0), none, nullptr, n, H / 2, W / 2, s);
+  // enc1: the first layer's gradients are FP32 throughout
+  k_pool_bwd_gz<<<grid(P * n * c0 / 8), 256, 0, s>>>(T_(u->gcat1, c1 + c0, c1), T_(u->gp1, c0),
+                                                     T_(u->cat1, c1 + c0, c1), ga, n, H, W, c0);
+  layer_backward(u, T_(u->e1a, c0), ga, L[1], T_(u->g1a, c0), none, nullptr, n, H, W, s);
+  k_wgrad_first<<<(unsigned)std::min<long long>((P * n + 127) / 128, 152 * 3), 256, 0, s>>>(
+      u->x, T_(u->g1a, c0), T_(u->e1a, c0), u->g + L[0].w_off, u->g + L[0].b_off, n, H, W);
+  count_launches(8);
 }
 
 cudaError_t refresh_bf16_weights(ashrt_unet* u, cudaStream_t s) {
@@ -1389,26 +1451,17 @@ ashrt_status ashrt_unet_create(ashrt_unet** out, int H, int W, int out_channels,
   A(&u->d1a, P0 * c0);
   A(&u->d1b, P0 * c0);
   A(&u->y, P0 * out_channels);
-  A(&u->gy, P0 * out_channels);
+  if (out_channels > 48) A(&u->ynhwc, P0 * out_channels);   // head not on the tcgen05 kernel
   A(&u->g1a, P0 * c0);
   A(&u->gcat1, P0 * (c1 + c0));
   A(&u->gp1, P0 / 4 * c0);
-  A(&u->g2a, P0 / 4 * c1);
   A(&u->gcat2, P0 / 4 * (c2 + c1));
   A(&u->gp2, P0 / 16 * c1);
-  A(&u->g3a, P0 / 16 * c2);
   A(&u->gcat3, P0 / 16 * (c3 + c2));
   A(&u->gp3, P0 / 64 * c2);
-  A(&u->gba, P0 / 64 * c3);
-  A(&u->gbb, P0 / 64 * c3);
-  A(&u->gd3a, P0 / 16 * c2);
-  A(&u->gd3b, P0 / 16 * c2);
-  A(&u->gd2a, P0 / 4 * c1);
-  A(&u->gd2b, P0 / 4 * c1);
-  A(&u->gd1a, P0 * c0);
-  A(&u->gd1b, P0 * c0);
   A(&u->rms, max_batch);
   A(&u->rmsacc, max_batch);
+  A(&u->gza, P0 * c0);
   A(&u->gzb, P0 * c0);
   A(&u->err, 1);
   A(&u->lam, out_channels);
@@ -1512,12 +1565,12 @@ ashrt_status ashrt_unet_forward(ashrt_unet* u, const float* x, float* y, int n, 
   compute_rms(u, x, per, n, s);
   k_pack_in<<<grid1d(per * n), 256, 0, s>>>(x, u->rms, u->x, per, n);
   count_launches(1);
-  net_forward(u, n, s, y);
+  HeadOut head = head_planar(u, y);
   if (rescale) {
-    k_rescale_out<<<grid1d(per * u->cout * n), 256, 0, s>>>(y, u->rms, per, u->cout, n,
-                                                           0.5f * (p - 2.f));
-    count_launches(1);
+    head.rms = u->rms;
+    head.wr_pow = 0.5f * (p - 2.f);
   }
+  net_forward(u, n, s, head);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_error("ashrt_unet_forward: %s", cudaGetErrorString(e));
@@ -1551,11 +1604,8 @@ ashrt_status ashrt_unet_train_step(ashrt_unet* u, const float* x, const float* t
   compute_rms(u, x, per, n, s);
   k_pack_in<<<grid1d(per * n), 256, 0, s>>>(x, u->rms, u->x, per, n);
   count_launches(1);
-  net_forward(u, n, s);
-  k_mse<<<grid1d(per * u->cout * n), 256, 0, s>>>(u->y, target, u->lam, u->gy, per, u->cout, n,
-                                                  u->loss);
-  count_launches(1);
-  net_backward(u, n, s);
+  net_forward(u, n, s, head_planar(u, u->y));
+  net_backward(u, target, n, s);
   if (lr > 0.f) {
     u->adam_t += 1;
     const float b1 = 0.9f, b2 = 0.999f;
@@ -1616,10 +1666,14 @@ ashrt_status ashrt_unet_predict(ashrt_unet* u, const float* x, float* m0, float*
   compute_rms(u, x, per, n, s);
   k_pack_in<<<grid1d(per * n), 256, 0, s>>>(x, u->rms, u->x, per, n);
   count_launches(1);
-  net_forward(u, n, s, u->y);
-  k_predict_out<<<grid1d(per * n), 256, 0, s>>>(u->y, u->rms, m0, wr0, per, u->cout,
-                                                          n, 0.5f * (p - 2.f));
-  count_launches(1);
+  HeadOut head;
+  head.main = m0;
+  head.main_n = (u->cout - 1) * per;
+  head.last = wr0;
+  head.last_n = per;
+  head.rms = u->rms;
+  head.wr_pow = 0.5f * (p - 2.f);
+  net_forward(u, n, s, head);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_error("ashrt_unet_predict: %s", cudaGetErrorString(e));
