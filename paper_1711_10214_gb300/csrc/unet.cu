@@ -9,9 +9,8 @@
 // gather [nx][nt] is an nx x nt image) with a per-tensor pixel stride and
 // channel offset, so skip connections are written straight into the channel
 // slice of the concatenation buffer they feed.  Convolution weights are kept
-// in FP32 "OIHW" order (the reference's order) and converted every step to a
-// BF16 [tap][ci][co] copy (forward) and a flipped, transposed [tap][co][ci]
-// copy (gradient with respect to the input).
+// in FP32 "OIHW" order (the reference's order) and converted every step to the
+// BF16 copies that the layer's kernels read (WCopies).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -267,8 +266,11 @@ __global__ void __launch_bounds__(256) k_pool_bwd_gz(Tensor g, Tensor gpool, Ten
 // own copy of gw: lane (ci, half) owns channels half, half + 2, ..  What bounds it
 // is HBM (y, t and the 16-channel maps once): 8 images 256 x 1024, 25 channels,
 // separate loss, weight- and input-gradient kernels 458 + 382 + 198 us and a mask
-// pass, this one see k_head_bwd's row in the launch list.
-constexpr int kHeadPix = 128, kHeadCh = 32;
+// pass, this one 267 (with the loss in FP64, three operations per element, 504).
+// WS: the head's weights (FP32) are in shared memory; else (very many channels) read
+// from global memory.
+constexpr int kHeadPix = 128, kHeadCh = 32, kHeadMaxShared = 1024;
+template <bool WS>
 __global__ void __launch_bounds__(kHeadPix) k_head_bwd(const float* __restrict__ y,
                                                        const float* __restrict__ t,
                                                        const float* __restrict__ lam,
@@ -280,7 +282,10 @@ __global__ void __launch_bounds__(kHeadPix) k_head_bwd(const float* __restrict__
   __shared__ __align__(16) float gys[kHeadCh][LD];
   __shared__ __align__(16) float as[16][LD];
   __shared__ double red[kHeadPix / 32];
+  extern __shared__ __align__(16) float wsh[];   // the head's weights [C][16]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (WS)
+    for (int i = tid; i < C * 16; i += kHeadPix) wsh[i] = __bfloat162float(w[i]);
   const int cb = blockIdx.y * kHeadCh, ci = lane & 15, half = lane >> 4;
   const bool first = blockIdx.y == 0;
   const double inv = 1.0 / ((double)P * N);
@@ -312,19 +317,39 @@ __global__ void __launch_bounds__(kHeadPix) k_head_bwd(const float* __restrict__
     const float* yp = y + n * C * P + p;
     const float* tp = t + n * C * P + p;
     const int c0 = first ? 0 : cb, c1 = first ? C : min(C, cb + kHeadCh);
-#pragma unroll 5
-    for (int c = c0; c < c1; ++c) {
-      const float l = __ldg(lam + c);
-      const float e = ok ? __ldg(yp + (long long)c * P) - __ldg(tp + (long long)c * P) : 0.f;
-      const float g = inv2 * l * e;
-      if (c >= cb && c < cb + kHeadCh) gys[c - cb][tid] = g;
-      if (first) {
-        loss2.add(l, e);
-        __align__(16) bf16 wv[16];
-        *(uint4*)wv = __ldg((const uint4*)(w + c * 16));
-        *(uint4*)(wv + 8) = __ldg((const uint4*)(w + c * 16 + 8));
+    for (int cc = c0; cc < c1; cc += 8) {       // eight channels' loads in flight
+      float yv[8], tv[8];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) gd[j] = fmaf(g, __bfloat162float(wv[j]), gd[j]);
+      for (int k = 0; k < 8; ++k) {
+        const bool in = ok && cc + k < c1;
+        yv[k] = in ? __ldg(yp + (long long)(cc + k) * P) : 0.f;
+        tv[k] = in ? __ldg(tp + (long long)(cc + k) * P) : 0.f;
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int c = cc + k;
+        if (c >= c1) break;
+        const float l = __ldg(lam + c), e = yv[k] - tv[k];
+        const float g = inv2 * l * e;
+        if (c >= cb && c < cb + kHeadCh) gys[c - cb][tid] = g;
+        if (first) {
+          loss2.add(l, e);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            float4 wv;
+            if (WS) {
+              wv = *(const float4*)(wsh + c * 16 + 4 * j);
+            } else {
+              const bf16* wg = w + c * 16 + 4 * j;
+              wv = make_float4(__bfloat162float(wg[0]), __bfloat162float(wg[1]),
+                               __bfloat162float(wg[2]), __bfloat162float(wg[3]));
+            }
+            gd[4 * j] = fmaf(g, wv.x, gd[4 * j]);
+            gd[4 * j + 1] = fmaf(g, wv.y, gd[4 * j + 1]);
+            gd[4 * j + 2] = fmaf(g, wv.z, gd[4 * j + 2]);
+            gd[4 * j + 3] = fmaf(g, wv.w, gd[4 * j + 3]);
+          }
+        }
       }
     }
     if (first && ok) {
@@ -453,20 +478,48 @@ __global__ void k_adam(float* w, const float* g, float* m, float* v, long long n
   }
 }
 
-// FP32 OIHW master -> BF16 [tap][ci][co] (forward, CUDA cores), flipped
-// [tap'][co][ci] (input gradient, CUDA cores), [tap][co][ci] (forward, tensor
-// cores) and flipped [tap'][ci][co] (input gradient, tensor cores)
-__global__ void k_wconv(const float* w, bf16* wf, bf16* wt, bf16* wn, bf16* wtn, int co_n, int ci_n,
-                        int K) {
+// The BF16 copies of a layer's FP32 OIHW master weights that its kernels read
+// (null where none does): wf [tap][ci][co] (first layer), wt [tap][co][ci] with the
+// taps flipped (head backward), wn [tap][co][ci] (the mma.sync head), and for the
+// tcgen05 convolutions wp (forward) and wtp (input gradient: channels exchanged, taps
+// flipped) in the order in which they lie in shared memory, one contiguous block per
+// output-channel tile and chunk of 16 input channels (see tc_weight).
+struct WCopies {
+  bf16 *wf = nullptr, *wt = nullptr, *wn = nullptr, *wp = nullptr, *wtp = nullptr;
+  int nt_p = 0, nt_t = 0;       // output-channel tiles of wp and wtp
+};
+// [tile][chunk][tap][channel octet][NT outputs][8 inputs] of weight (out o, in i)
+__host__ __device__ __forceinline__ long long tc_weight(int o, int i, int tap, int nch, int taps,
+                                                        int NT) {
+  return (((((long long)(o / NT) * nch + i / 16) * taps + tap) * 2 + (i / 8) % 2) * NT + o % NT) * 8 +
+         i % 8;
+}
+__global__ void k_wconv(const float* w, WCopies c, int co_n, int ci_n, int K) {
   const int total = co_n * ci_n * K * K;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
     const int kx = i % K, ky = (i / K) % K, ci = (i / (K * K)) % ci_n, co = i / (K * K * ci_n);
     const int tap = ky * K + kx, tapf = (K * K - 1) - tap;
     const bf16 b = __float2bfloat16(w[i]);
-    wf[((long long)tap * ci_n + ci) * co_n + co] = b;
-    wt[((long long)tapf * co_n + co) * ci_n + ci] = b;
-    wn[((long long)tap * co_n + co) * ci_n + ci] = b;
-    wtn[((long long)tapf * ci_n + ci) * co_n + co] = b;
+    if (c.wf) c.wf[((long long)tap * ci_n + ci) * co_n + co] = b;
+    if (c.wt) c.wt[((long long)tapf * co_n + co) * ci_n + ci] = b;
+    if (c.wn) c.wn[((long long)tap * co_n + co) * ci_n + ci] = b;
+    if (c.wp) c.wp[tc_weight(co, ci, tap, ci_n / 16, K * K, c.nt_p)] = b;
+    if (c.wtp) c.wtp[tc_weight(ci, co, tapf, co_n / 16, K * K, c.nt_t)] = b;
+  }
+}
+
+// Output-channel tile of the tcgen05 convolution with `cout` outputs (0: none is
+// compiled).
+int tc_tile(int K, int cout) {
+  const int nt = (cout + 15) / 16 * 16;
+  if (K == 1) return nt <= 48 ? nt : 0;
+  switch (nt) {
+    case 16: return 16;
+    case 48: case 144: return 48;
+    case 64: return 64;
+    case 96: case 288: return 96;
+    case 192: return 192;
+    default: return 0;
   }
 }
 
@@ -604,7 +657,7 @@ __global__ void k_targets(const float* m, const float* wr, const float* rms, flo
 struct Layer {
   int ci, co, k;
   long long w_off, b_off;   // into the flat parameter buffer
-  bf16 *wf = nullptr, *wt = nullptr, *wn = nullptr, *wtn = nullptr;
+  WCopies c;
 };
 
 int grid1d(long long n) {
@@ -663,13 +716,24 @@ Tensor T_(void* p, int ps, int off = 0) {
 //   A: [dy][2 channel octets][130 pixels][8 channels]  (a tap's A operand
 //      starts dx pixels in: rows 16 B apart, next 8 pixels at +128 B = SBO,
 //      next channel octet at +130 x 16 B = LBO)
-//   B: [tap][2 octets][NT channels][8 input channels]  (SBO 128 B, LBO NT x 16 B)
-// with cp.async into one of two stages, so that the copies of the next chunk
-// overlap the MMAs of the current one; one thread issues the taps' MMAs and
-// commits them to the stage's mbarrier, which is waited on (bounded) before
-// that stage is refilled.  The epilogue reads the accumulators with tcgen05.ld
-// (warps w and w + 4: lanes 32 (w mod 4)..+31, alternate column groups) and
-// fuses bias, ReLU and the store.
+//   B: [tap][2 octets][NT channels][8 input channels]  (SBO 128 B, LBO NT x 16 B),
+// B once per CTA where all chunks' weights fit in 48 KB.
+// One persistent CTA per SM walks over its tiles with three roles:
+//   warps 8..11 copy (cp.async) the chunks of one tile after the other into a ring
+//     of three to six stages, three chunks ahead of the one they hand over;
+//   one thread of warp 12 issues the taps' MMAs of each chunk and commits them to
+//     the stage's "empty" barrier, and a tile's last chunk to "tile done";
+//   warps 0..7 read a finished tile's accumulators with tcgen05.ld (warps w and w + 4:
+//     lanes 32 (w mod 4)..+31, alternate column groups), fuse bias, ReLU or the
+//     mask and store, while the next tile accumulates in the other half of TMEM.
+// Every wait is bounded; one that runs out ends its role, then the others', and
+// sets the error flag.  What bounds a layer is the tensor pipe's reads of A (4 KB
+// per MMA, 32 cycles: with 16 to 96 columns a tap multiplies no longer than that).
+// 16 images 256 x 1024, the thirteen 3x3 layers and the head: with one tile per
+// CTA, two to three CTAs per SM and two stages the copies (800 us), MMAs (540) and
+// stores (440) ran one after the other, 2190 us; so 1280 us.  Weights in their own
+// order (32-byte pieces, the same ones for every SM at once) held the wide layers
+// back: packed blocks took the 192-channel layers from 301 to 134 us.
 __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
   return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
          ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);   // version 1, no swizzle
@@ -722,7 +786,7 @@ __global__ void k_unpack_out(const float* y, HeadOut h, long long P, int C, int 
 
 struct TcConvArgs {
   Tensor in;             // bf16 NHWC slice, ps and off multiples of 8
-  const bf16* w;         // [K*K][Cout][Cin]
+  const bf16* w;         // as they lie in shared memory (tc_weight)
   const float* bias;     // [Cout]
   Tensor out;            // bf16 or fp32 NHWC slice
   int N, H, W, Cin, Cout, relu;
@@ -732,246 +796,303 @@ struct TcConvArgs {
   HeadOut head;          // planar: where the outputs go
 };
 
+// (L2::128B: a pixel's other channels, in the same line, are copied next)
+__device__ __forceinline__ void cp16_line(void* dst, const void* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16, %2;\n" ::"r"(smem_addr(dst)),
+               "l"(src), "r"(valid ? 16 : 0)
+               : "memory");
+}
+
 __device__ __forceinline__ void cp16(void* dst, const void* src, bool valid) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem_addr(dst)), "l"(src),
                "r"(valid ? 16 : 0)
                : "memory");
 }
 
+template <int K, int NT, int RR>
+struct TcTile {
+  static constexpr int R = K / 2, PW = 128 + 2 * R, TAPS = K * K, ROWS = RR + 2 * R;
+  static constexpr int DS = (NT + 31) / 32 * 32;        // TMEM columns per output row
+  static constexpr int NCOL = RR * DS <= 32 ? 32 : RR * DS <= 64 ? 64 : RR * DS <= 128 ? 128 : 256;
+  static constexpr uint32_t A_PLANE = PW * 16, B_PLANE = NT * 16;       // bytes per channel octet
+  static constexpr uint32_t A_BYTES = ROWS * 2 * A_PLANE, B_BYTES = TAPS * 2 * B_PLANE;
+  // the weights of all channel chunks stay in shared memory where they are small
+  static bool resident(int nch) { return nch * B_BYTES <= 48 * 1024; }
+  // stages of the ring in about 200 KB, three to six
+  static int stages(int nch) {
+    const bool res = resident(nch);
+    const int n = (int)((205 * 1024 - (res ? nch * B_BYTES : 0)) / (A_BYTES + (res ? 0 : B_BYTES)));
+    return n > 6 ? 6 : n;
+  }
+  // more than half an SM's, so that one CTA is resident (it holds up to all of TMEM)
+  static size_t smem(int nch) {
+    const size_t n = (size_t)stages(nch) * (A_BYTES + (resident(nch) ? 0 : B_BYTES)) +
+                     (resident(nch) ? nch * B_BYTES : 0) + 256;
+    return n < 120 * 1024 ? 120 * 1024 : n;
+  }
+};
+
+constexpr int kTcEpi = 256, kTcCopy = 128, kTcThreads = kTcEpi + kTcCopy + 32;
+constexpr int kTcAhead = 2;   // chunks copied beyond the one handed over (stages >= kTcAhead + 1)
+
+__device__ __forceinline__ void tc_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void tc_commit(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+          smem_addr(bar))
+      : "memory");
+}
+
 template <int K, int NT, int RR, typename TO>
-__global__ void __launch_bounds__(256) k_conv_tc(TcConvArgs a) {
-  constexpr int R = K / 2, PW = 128 + 2 * R, TAPS = K * K, T = 256, ROWS = RR + 2 * R;
-  constexpr int DS = (NT + 31) / 32 * 32;        // TMEM columns per output row
-  constexpr int NCOL = RR * DS <= 32 ? 32 : RR * DS <= 64 ? 64 : RR * DS <= 128 ? 128 : 256;
+__global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(TcConvArgs a, int n_tiles, int stages,
+                                                           int b_resident) {
+  using S = TcTile<K, NT, RR>;
+  constexpr int R = S::R, TAPS = S::TAPS, ROWS = S::ROWS, DS = S::DS, NCOL = S::NCOL;
+  constexpr uint32_t A_PLANE = S::A_PLANE, B_PLANE = S::B_PLANE;
+  constexpr uint32_t A_BYTES = S::A_BYTES, B_BYTES = S::B_BYTES;
   static_assert(RR * DS <= 256, "TMEM tile");
-  constexpr uint32_t A_PLANE = PW * 16, B_PLANE = NT * 16;       // bytes per channel octet
-  constexpr uint32_t A_BYTES = ROWS * 2 * A_PLANE, B_BYTES = TAPS * 2 * B_PLANE;
   constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NT >> 3) << 17) |
                              ((uint32_t)(128 >> 4) << 24);        // F32 += BF16 x BF16, M 128
   extern __shared__ __align__(128) unsigned char smt[];
-  // two stages of [A | B]; then two mbarriers (one per stage) and the TMEM slot
-  uint64_t* bar = (uint64_t*)(smt + 2 * (A_BYTES + B_BYTES));
-  uint32_t* tslot = (uint32_t*)(bar + 2);
+  const int nch = a.Cin / 16;
+  unsigned char* const Bbase = smt + stages * A_BYTES;
+  uint64_t* full = (uint64_t*)(Bbase + (b_resident ? nch : stages) * B_BYTES);
+  uint64_t *empty = full + 6, *tfull = full + 12, *tempty = full + 14;
+  uint32_t* tslot = (uint32_t*)(full + 16);
+  __shared__ __align__(16) float sbias[NT];
   const int tid = threadIdx.x, warp = tid >> 5;
   const int xt = (a.W + 127) / 128, yt = (a.H + RR - 1) / RR;
-  const int x0 = (blockIdx.x % xt) * 128;
-  const int rb = blockIdx.x / xt;                 // n * yt + row block
-  const int n = rb / yt, y0 = (rb % yt) * RR;
   const int co0 = blockIdx.y * NT;                // output-channel tile
-  const bf16* in = (const bf16*)a.in.p;
-  const int nch = a.Cin / 16;
-
+  if (tid < NT) sbias[tid] = a.bias && co0 + tid < a.Cout ? a.bias[co0 + tid] : 0.f;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                      smem_addr(tslot)),
-                 "r"((uint32_t)NCOL));
+                 "r"((uint32_t)(2 * NCOL)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
   }
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_addr(bar)));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_addr(bar + 1)));
+    for (int i = 0; i < 16; ++i)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(full + i)),
+                   "r"(i < 6 ? kTcCopy : i < 14 ? 1 : kTcEpi));
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = *tslot;
+  bool ok = true;
 
-  // asynchronous copies of channel chunk c into stage st (zero-filled outside the
-  // image): two threads per pixel, one 16-byte octet each, row by row; the 2 R
-  // halo pixels at the row's end by the first threads.  What a thread copies is
-  // the same in every chunk but for the channel, so its addresses are formed once.
-  const int sp = tid >> 1, so = tid & 1;
-  const bool okx = x0 + sp - R >= 0 && x0 + sp - R < a.W;
-  const long long rstride = (long long)a.W * a.in.ps;
-  const bf16* src0 = in + (((long long)n * a.H + y0 - R) * a.W + x0 + sp - R) * a.in.ps +
-                     a.in.off + 8 * so;
-  const int hr = tid >> 2, hp = 128 + (sp & 1);            // halo row and pixel
-  const bool okh = R > 0 && tid < 4 * ROWS && x0 + hp - R < a.W && y0 + hr - R >= 0 &&
-                   y0 + hr - R < a.H;
-  const bf16* srch = src0 + (long long)hr * rstride + (long long)(hp - sp) * a.in.ps;
-  auto stage = [&](int c, int st) {
-    unsigned char* As = smt + st * (A_BYTES + B_BYTES);
-    unsigned char* Bs = As + A_BYTES;
-    const int ci0 = c * 16;
+  if (warp >= kTcEpi / 32 && warp < (kTcEpi + kTcCopy) / 32) {
+    // ---- copies: two threads per pixel, one 16-byte octet each (zero-filled
+    // outside the image); the 2 R halo pixels at a row's end by the first threads
+    const int t = tid - kTcEpi, sp = t >> 1, so = t & 1, hr = t >> 2, hp = 128 + (sp & 1);
+    const bf16* in = (const bf16*)a.in.p;
+    const long long rstride = (long long)a.W * a.in.ps;
+    const uint4* wsrc = (const uint4*)a.w + (size_t)blockIdx.y * nch * (B_BYTES / 16);
+    auto stage_b = [&](int c, unsigned char* Bs) {
+      const uint4* src = wsrc + (size_t)c * (B_BYTES / 16);
+#pragma unroll 6
+      for (int e = t; e < (int)(B_BYTES / 16); e += kTcCopy) cp16(Bs + e * 16, src + e, true);
+    };
+    // hands over stage st: its copies are complete and visible to the MMAs
+    auto hand_over = [&](int st) {
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      tc_arrive(full + st);
+    };
+    if (b_resident)
+      for (int c = 0; c < nch; ++c) stage_b(c, Bbase + c * B_BYTES);
+    int st = 0, out = 0, n = 0;              // stage of this step, of the next hand-over; steps
+    uint32_t phase = 1;                      // parity the stage's previous use leaves
+    for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+      const int x0 = (tile % xt) * 128 - R, rb = tile / xt, y0 = (rb % yt) * RR - R;
+      const bf16* src = in + (((long long)(rb / yt) * a.H + y0) * a.W + x0) * a.in.ps + a.in.off + 8 * so;
+      for (int c = 0; c < nch; ++c, src += 16, ++n) {
+        if (!(ok = tc_wait(empty + st, phase))) break;
+        unsigned char* As = smt + st * A_BYTES;
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r) {
-      const bool ok = okx && y0 + r - R >= 0 && y0 + r - R < a.H;
-      cp16(As + (r * 2 + so) * A_PLANE + sp * 16, ok ? src0 + r * rstride + ci0 : in, ok);
-    }
-    if (R > 0 && tid < 4 * ROWS)
-      cp16(As + (hr * 2 + so) * A_PLANE + hp * 16, okh ? srch + ci0 : in, okh);
+        for (int half = 0; half < 2; ++half) {
+          const int px = sp + 64 * half;
+          const bool okx = x0 + px >= 0 && x0 + px < a.W;
+          const bf16* s0 = src + (long long)px * a.in.ps;
 #pragma unroll
-    for (int i = 0; i < (TAPS * NT + 127) / 128; ++i) {
-      const int e = sp + 128 * i, c = e % NT, tap = e / NT;
-      if (e < TAPS * NT) {
-        const bool ok = co0 + c < a.Cout;
-        const bf16* src = ok ? a.w + ((long long)tap * a.Cout + co0 + c) * a.Cin + ci0 + 8 * so : a.w;
-        cp16(Bs + (tap * 2 + so) * B_PLANE + c * 16, src, ok);
-      }
-    }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-  };
-
-  uint32_t uses[2] = {0u, 0u};   // completed MMA batches per stage (barrier parity)
-  bool failed = false;
-  stage(0, 0);
-  for (int c = 0; c < nch; ++c) {
-    const int st = c & 1;
-    if (c + 1 < nch) {
-      // stage c+1 goes into the buffers of chunk c-1: wait for its MMAs first
-      if (c >= 1) {
-        const bool ok = tc_wait(bar + (st ^ 1), uses[st ^ 1] & 1u);
-        uses[st ^ 1] += 1u;
-        if (__syncthreads_or(!ok)) {
-          failed = true;
-          break;
+          for (int r = 0; r < ROWS; ++r) {
+            const bool in_img = okx && y0 + r >= 0 && y0 + r < a.H;
+            cp16_line(As + (r * 2 + so) * A_PLANE + px * 16, in_img ? s0 + r * rstride : in, in_img);
+          }
+        }
+        if (R > 0 && t < 4 * ROWS) {
+          const bool in_img = x0 + hp < a.W && y0 + hr >= 0 && y0 + hr < a.H;
+          cp16_line(As + (hr * 2 + so) * A_PLANE + hp * 16,
+               in_img ? src + hr * rstride + (long long)hp * a.in.ps : in, in_img);
+        }
+        if (!b_resident) stage_b(c, Bbase + st * B_BYTES);
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+        if (n >= kTcAhead) {
+          asm volatile("cp.async.wait_group %0;\n" ::"n"(kTcAhead) : "memory");
+          hand_over(out);
+          out = out + 1 == stages ? 0 : out + 1;
+        }
+        if (++st == stages) {
+          st = 0;
+          phase ^= 1u;
         }
       }
-      stage(c + 1, st ^ 1);
-      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     }
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      const unsigned char* As = smt + st * (A_BYTES + B_BYTES);
-      const unsigned char* Bs = As + A_BYTES;
-#pragma unroll
-      for (int r = 0; r < RR; ++r) {
-#pragma unroll
-        for (int tap = 0; tap < TAPS; ++tap) {
-          const int dy = tap / K, dx = tap % K;
-          const uint64_t ad =
-              umma_desc(smem_addr(As + (r + dy) * 2 * A_PLANE + dx * 16), A_PLANE, 128);
-          const uint64_t bd = umma_desc(smem_addr(Bs + tap * 2 * B_PLANE), B_PLANE, 128);
-          const uint32_t acc = (c > 0 || tap > 0) ? 1u : 0u;
-          asm volatile(
-              "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-              " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-                  tmem + (uint32_t)(r * DS)),
-              "l"(ad), "l"(bd), "r"(IDESC), "r"(acc));
-        }
-      }
-      asm volatile(
-          "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-              smem_addr(bar + st))
-          : "memory");
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    for (int i = n < kTcAhead ? n : kTcAhead; i > 0 && ok; --i) {
+      hand_over(out);
+      out = out + 1 == stages ? 0 : out + 1;
     }
-  }
-  if (!failed) {
-    // the last batch's completion implies all earlier ones (same issuing thread)
-    const int st = (nch - 1) & 1;
-    const bool ok = tc_wait(bar + st, uses[st] & 1u);
-    if (__syncthreads_or(!ok)) failed = true;
-  }
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-
-  if (!failed) {
-    // epilogue: thread = pixel (TMEM lane of its warp quarter); warps w and
-    // w + 4 share lanes and split the (row, 16-column) groups
-    const int lane_base = (warp & 3) * 32;
-    const int xx = x0 + lane_base + (tid & 31);
-    TO* out = (TO*)a.out.p;
-    constexpr int G = NT / 16;
-    for (int gi = warp >> 2; gi < RR * G; gi += 2) {
-      const int r = gi / G, c0 = (gi % G) * 16;
-      uint32_t v[16];
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-          "%11, %12, %13, %14, %15}, [%16];\n"
-          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-            "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
-            "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-          : "r"(tmem + ((uint32_t)lane_base << 16) + (uint32_t)(r * DS + c0)));
-      asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-      const int y = y0 + r;
-      if (xx < a.W && y < a.H) {
-        const long long pix = ((long long)n * a.H + y) * a.W + xx;
-        const int cb = co0 + c0;                    // first output channel of the group
-        float f[16];
+  } else if (warp == (kTcEpi + kTcCopy) / 32) {
+    // ---- MMAs: one thread
+    if ((tid & 31) == 0) {
+      int st = 0, k = 0;
+      uint32_t phase = 0;
+      for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++k) {
+        // the accumulators' previous tile has been read
+        ok = tc_wait(tempty + (k & 1), ((k >> 1) & 1) ^ 1);
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        for (int c = 0; c < nch && ok; ++c) {
+          if (!(ok = tc_wait(full + st, phase))) break;
+          asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+          const uint32_t As = smem_addr(smt + st * A_BYTES);
+          const uint32_t Bs = smem_addr(Bbase + (b_resident ? c : st) * B_BYTES);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          f[j] = __uint_as_float(v[j]) + ((a.bias && cb + j < a.Cout) ? a.bias[cb + j] : 0.f);
-          if (a.relu) f[j] = fmaxf(f[j], 0.f);
-        }
-        const bool whole = cb + 16 <= a.Cout;
-        if (a.planar) {
-          // the stores of a warp are contiguous
-          const long long P = (long long)a.H * a.W, p = (long long)y * a.W + xx;
-          const float rms = a.head.rms ? a.head.rms[n] : 1.f;
+          for (int r = 0; r < RR; ++r) {
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            if (cb + j < a.Cout - 1) {
-              if (a.head.main)
-                a.head.main[n * a.head.main_n + (cb + j) * P + p] = a.head.rms ? f[j] * rms : f[j];
-            } else if (cb + j == a.Cout - 1 && a.head.last) {
-              a.head.last[n * a.head.last_n + p] =
-                  a.head.rms ? expf(f[j]) * powf(rms, a.head.wr_pow) : f[j];
+            for (int tap = 0; tap < TAPS; ++tap) {
+              const int dy = tap / K, dx = tap % K;
+              const uint64_t ad = umma_desc(As + (r + dy) * 2 * A_PLANE + dx * 16, A_PLANE, 128);
+              const uint64_t bd = umma_desc(Bs + tap * 2 * B_PLANE, B_PLANE, 128);
+              const uint32_t acc = (c > 0 || tap > 0) ? 1u : 0u;
+              asm volatile(
+                  "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                  " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
+                      tmem + (uint32_t)((k & 1) * NCOL + r * DS)),
+                  "l"(ad), "l"(bd), "r"(IDESC), "r"(acc));
             }
           }
-        } else if (sizeof(TO) == 2 && whole && ((a.out.ps | a.out.off) & 7) == 0) {
-          __align__(16) bf16 o[16];
-          if (a.mask.p) {
-            const uint4* mp = (const uint4*)((const bf16*)a.mask.p + pix * a.mask.ps + a.mask.off + cb);
-            __align__(16) bf16 m[16];
-            *(uint4*)m = mp[0];
-            *(uint4*)(m + 8) = mp[1];
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (__bfloat162float(m[j]) <= 0.f) f[j] = 0.f;
+          tc_commit(empty + st);
+          if (c + 1 == nch) tc_commit(tfull + (k & 1));
+          if (++st == stages) {
+            st = 0;
+            phase ^= 1u;
           }
-#pragma unroll
-          for (int j = 0; j < 16; ++j) o[j] = __float2bfloat16(f[j]);
-          bf16* dst = (bf16*)out + pix * a.out.ps + a.out.off + cb;
-          *(uint4*)dst = *(const uint4*)o;
-          *(uint4*)(dst + 8) = *(const uint4*)(o + 8);
-        } else if (sizeof(TO) == 4 && whole && ((a.out.ps | a.out.off) & 3) == 0) {
-          float4* dst = (float4*)((float*)out + pix * a.out.ps + a.out.off + cb);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) dst[q] = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (cb + j < a.Cout) st_f(out, pix * a.out.ps + a.out.off + cb + j, f[j]);
         }
       }
     }
-  } else if (tid == 0 && a.err) {
-    atomicExch(a.err, 1);
+  } else {
+    int k = 0;
+    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++k) {
+      const int x0 = (tile % xt) * 128, rb = tile / xt, n = rb / yt, y0 = (rb % yt) * RR;
+      const uint32_t tacc = tmem + (uint32_t)((k & 1) * NCOL);
+      ok = tc_wait(tfull + (k & 1), (k >> 1) & 1);
+      if (!__all_sync(0xffffffffu, ok)) {
+        ok = false;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+      // epilogue: thread = pixel (TMEM lane of its warp quarter); warps w and
+      // w + 4 share lanes and split the (row, 16-column) groups
+      const int lane_base = (warp & 3) * 32;
+      const int xx = x0 + lane_base + (tid & 31);
+      TO* out = (TO*)a.out.p;
+      constexpr int G = NT / 16;
+      for (int gi = warp >> 2; gi < RR * G; gi += 2) {
+        const int r = gi / G, c0 = (gi % G) * 16;
+        uint32_t v[16];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+            "%11, %12, %13, %14, %15}, [%16];\n"
+            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+              "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
+              "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+            : "r"(tacc + ((uint32_t)lane_base << 16) + (uint32_t)(r * DS + c0)));
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+        const int y = y0 + r;
+        if (xx < a.W && y < a.H) {
+          const long long pix = ((long long)n * a.H + y) * a.W + xx;
+          const int cb = co0 + c0;                    // first output channel of the group
+          float f[16];
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            f[j] = __uint_as_float(v[j]) + sbias[c0 + j];
+            if (a.relu) f[j] = fmaxf(f[j], 0.f);
+          }
+          const bool whole = cb + 16 <= a.Cout;
+          if (a.planar) {
+            // the stores of a warp are contiguous
+            const long long P = (long long)a.H * a.W, p = (long long)y * a.W + xx;
+            const float rms = a.head.rms ? a.head.rms[n] : 1.f;
+            float* o = a.head.main ? a.head.main + n * a.head.main_n + cb * P + p : nullptr;
+            float flast = 0.f;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              if (o && cb + j < a.Cout - 1) o[j * P] = a.head.rms ? f[j] * rms : f[j];
+              flast = cb + j == a.Cout - 1 ? f[j] : flast;
+            }
+            if (a.head.last && cb < a.Cout && cb + 16 >= a.Cout)
+              a.head.last[n * a.head.last_n + p] =
+                  a.head.rms ? expf(flast) * powf(rms, a.head.wr_pow) : flast;
+          } else if (sizeof(TO) == 2 && whole && ((a.out.ps | a.out.off) & 7) == 0) {
+            __align__(16) bf16 o[16];
+            if (a.mask.p) {
+              const uint4* mp = (const uint4*)((const bf16*)a.mask.p + pix * a.mask.ps + a.mask.off + cb);
+              __align__(16) bf16 m[16];
+              *(uint4*)m = mp[0];
+              *(uint4*)(m + 8) = mp[1];
+#pragma unroll
+              for (int j = 0; j < 16; ++j)
+                if (__bfloat162float(m[j]) <= 0.f) f[j] = 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) o[j] = __float2bfloat16(f[j]);
+            bf16* dst = (bf16*)out + pix * a.out.ps + a.out.off + cb;
+            *(uint4*)dst = *(const uint4*)o;
+            *(uint4*)(dst + 8) = *(const uint4*)(o + 8);
+          } else if (sizeof(TO) == 4 && whole && ((a.out.ps | a.out.off) & 3) == 0) {
+            float4* dst = (float4*)((float*)out + pix * a.out.ps + a.out.off + cb);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) dst[q] = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              if (cb + j < a.Cout) st_f(out, pix * a.out.ps + a.out.off + cb + j, f[j]);
+          }
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+      tc_arrive(tempty + (k & 1));
+    }
   }
+  if (!ok && a.err) atomicExch(a.err, 1);
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
-                 "r"((uint32_t)NCOL));
+                 "r"((uint32_t)(2 * NCOL)));
   }
 }
 
 template <int K, int NT, int RR, typename TO>
 void conv_tc_v(const TcConvArgs& a, cudaStream_t s) {
-  constexpr int R = K / 2, PW = 128 + 2 * R, ROWS = RR + 2 * R, DS = (NT + 31) / 32 * 32;
-  constexpr int NCOL = RR * DS <= 32 ? 32 : RR * DS <= 64 ? 64 : RR * DS <= 128 ? 128 : 256;
-  // at most 512 / NCOL CTAs per SM may hold TMEM at once: request enough
-  // shared memory that no more are resident (228 KB per SM, 1 KB reserved
-  // per CTA), so that no CTA waits in tcgen05.alloc
-  const size_t need = 2 * ((size_t)ROWS * 2 * PW * 16 + (size_t)K * K * 2 * NT * 16) + 32;
-  const size_t floor_b = 233472 / (512 / NCOL + 1);
-  const size_t smem = std::max(need, floor_b);
-  static bool attr = false;
-  if (!attr) {
+  using S = TcTile<K, NT, RR>;
+  const int nch = a.Cin / 16;
+  const size_t smem = S::smem(nch);
+  static size_t attr = 0;
+  if (smem > attr) {
     cudaFuncSetAttribute(k_conv_tc<K, NT, RR, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
-    attr = true;
+    attr = smem;
   }
-  dim3 grid((unsigned)((long long)a.N * ((a.H + RR - 1) / RR) * ((a.W + 127) / 128)),
-            (unsigned)((a.Cout + NT - 1) / NT));
-  k_conv_tc<K, NT, RR, TO><<<grid, 256, smem, s>>>(a);
+  const int tiles = a.N * ((a.H + RR - 1) / RR) * ((a.W + 127) / 128);
+  const int gy = (a.Cout + NT - 1) / NT;
+  const int gx = std::min(tiles, std::max(1, 152 / gy));   // one CTA per SM
+  k_conv_tc<K, NT, RR, TO><<<dim3(gx, gy), kTcThreads, smem, s>>>(a, tiles, S::stages(nch),
+                                                                 S::resident(nch) ? 1 : 0);
   count_launches(1);
 }
 
@@ -998,23 +1119,22 @@ bool conv_tc(Tensor in, const bf16* w, const float* bias, Tensor out, int N, int
   a.Cout = Cout;
   a.relu = relu;
   a.err = err;
-  const int nt = (Cout + 15) / 16 * 16;
   if constexpr (K == 3) {
     // output rows per CTA: the staged input rows serve RR outputs (TMEM:
     // RR x NT <= 256); wider outputs are split into NT-channel tiles
-    switch (nt) {
+    switch (tc_tile(K, Cout)) {
       case 16: conv_tc_v<3, 16, 4, TO>(a, s); return true;
-      case 48: case 144: conv_tc_v<3, 48, 4, TO>(a, s); return true;
+      case 48: conv_tc_v<3, 48, 4, TO>(a, s); return true;
       case 64: conv_tc_v<3, 64, 4, TO>(a, s); return true;
-      case 96: case 288: conv_tc_v<3, 96, 2, TO>(a, s); return true;
+      case 96: conv_tc_v<3, 96, 2, TO>(a, s); return true;
       case 192: conv_tc_v<3, 192, 1, TO>(a, s); return true;
       default: return false;
     }
   } else {
-    switch (nt) {
-      case 16: conv_tc_v<1, 16, 1, TO>(a, s); return true;
-      case 32: conv_tc_v<1, 32, 1, TO>(a, s); return true;
-      case 48: conv_tc_v<1, 48, 1, TO>(a, s); return true;
+    switch (tc_tile(K, Cout)) {
+      case 16: conv_tc_v<1, 16, 4, TO>(a, s); return true;
+      case 32: conv_tc_v<1, 32, 4, TO>(a, s); return true;
+      case 48: conv_tc_v<1, 48, 4, TO>(a, s); return true;
       default: return false;
     }
   }
@@ -1040,8 +1160,7 @@ void conv_mma_v(const MmaConvArgs& a, cudaStream_t s) {
 // output-channel tile from the layer's sizes.
 template <int K, typename TO>
 void conv_mma(Tensor in, const bf16* w, const float* bias, Tensor out, int N, int H, int W,
-              int Cin, int Cout, int relu, cudaStream_t s, int* err = nullptr) {
-  if (conv_tc<K, TO>(in, w, bias, out, N, H, W, Cin, Cout, relu, err, s)) return;
+              int Cin, int Cout, int relu, cudaStream_t s) {
   MmaConvArgs a;
   a.in = in;
   a.w = w;
@@ -1100,33 +1219,33 @@ void net_forward(ashrt_unet* u, int n, cudaStream_t s, const HeadOut& head) {
   auto B = [&](int i) { return u->w + L[i].b_off; };
   auto grid = [&](long long cnt) { return grid1d(cnt); };
   // encoder
-  k_conv_first<<<grid((long long)n * H * W / 4), 256, 0, s>>>(u->x, L[0].wf, B(0), T_(u->e1a, c0), n,
+  k_conv_first<<<grid((long long)n * H * W / 4), 256, 0, s>>>(u->x, L[0].c.wf, B(0), T_(u->e1a, c0), n,
                                                           H, W, 1);
-  conv_mma<3, bf16>(T_(u->e1a, c0), L[1].wn, B(1), T_(u->cat1, c1 + c0, c1), n, H, W, c0, c0, 1, s, u->err);
+  conv_tc<3, bf16>(T_(u->e1a, c0), L[1].c.wp, B(1), T_(u->cat1, c1 + c0, c1), n, H, W, c0, c0, 1, u->err, s);
   k_pool<<<grid((long long)n * H * W / 4 * c0 / 8), 256, 0, s>>>(T_(u->cat1, c1 + c0, c1), T_(u->p1, c0), n, H, W, c0);
-  conv_mma<3, bf16>(T_(u->p1, c0), L[2].wn, B(2), T_(u->e2a, c1), n, H / 2, W / 2, c0, c1, 1, s, u->err);
-  conv_mma<3, bf16>(T_(u->e2a, c1), L[3].wn, B(3), T_(u->cat2, c2 + c1, c2), n, H / 2, W / 2, c1, c1, 1, s, u->err);
+  conv_tc<3, bf16>(T_(u->p1, c0), L[2].c.wp, B(2), T_(u->e2a, c1), n, H / 2, W / 2, c0, c1, 1, u->err, s);
+  conv_tc<3, bf16>(T_(u->e2a, c1), L[3].c.wp, B(3), T_(u->cat2, c2 + c1, c2), n, H / 2, W / 2, c1, c1, 1, u->err, s);
   k_pool<<<grid((long long)n * H * W / 16 * c1 / 8), 256, 0, s>>>(T_(u->cat2, c2 + c1, c2), T_(u->p2, c1), n, H / 2, W / 2, c1);
-  conv_mma<3, bf16>(T_(u->p2, c1), L[4].wn, B(4), T_(u->e3a, c2), n, H / 4, W / 4, c1, c2, 1, s, u->err);
-  conv_mma<3, bf16>(T_(u->e3a, c2), L[5].wn, B(5), T_(u->cat3, c3 + c2, c3), n, H / 4, W / 4, c2, c2, 1, s, u->err);
+  conv_tc<3, bf16>(T_(u->p2, c1), L[4].c.wp, B(4), T_(u->e3a, c2), n, H / 4, W / 4, c1, c2, 1, u->err, s);
+  conv_tc<3, bf16>(T_(u->e3a, c2), L[5].c.wp, B(5), T_(u->cat3, c3 + c2, c3), n, H / 4, W / 4, c2, c2, 1, u->err, s);
   k_pool<<<grid((long long)n * H * W / 64 * c2 / 8), 256, 0, s>>>(T_(u->cat3, c3 + c2, c3), T_(u->p3, c2), n, H / 4, W / 4, c2);
-  conv_mma<3, bf16>(T_(u->p3, c2), L[6].wn, B(6), T_(u->ba, c3), n, H / 8, W / 8, c2, c3, 1, s, u->err);
-  conv_mma<3, bf16>(T_(u->ba, c3), L[7].wn, B(7), T_(u->bb, c3), n, H / 8, W / 8, c3, c3, 1, s, u->err);
+  conv_tc<3, bf16>(T_(u->p3, c2), L[6].c.wp, B(6), T_(u->ba, c3), n, H / 8, W / 8, c2, c3, 1, u->err, s);
+  conv_tc<3, bf16>(T_(u->ba, c3), L[7].c.wp, B(7), T_(u->bb, c3), n, H / 8, W / 8, c3, c3, 1, u->err, s);
   // decoder
   k_up<<<grid((long long)n * H * W / 16 * c3 / 8), 256, 0, s>>>(T_(u->bb, c3), T_(u->cat3, c3 + c2, 0), n, H / 4, W / 4, c3);
-  conv_mma<3, bf16>(T_(u->cat3, c3 + c2), L[8].wn, B(8), T_(u->d3a, c2), n, H / 4, W / 4, c3 + c2, c2, 1, s, u->err);
-  conv_mma<3, bf16>(T_(u->d3a, c2), L[9].wn, B(9), T_(u->d3b, c2), n, H / 4, W / 4, c2, c2, 1, s, u->err);
+  conv_tc<3, bf16>(T_(u->cat3, c3 + c2), L[8].c.wp, B(8), T_(u->d3a, c2), n, H / 4, W / 4, c3 + c2, c2, 1, u->err, s);
+  conv_tc<3, bf16>(T_(u->d3a, c2), L[9].c.wp, B(9), T_(u->d3b, c2), n, H / 4, W / 4, c2, c2, 1, u->err, s);
   k_up<<<grid((long long)n * H * W / 4 * c2 / 8), 256, 0, s>>>(T_(u->d3b, c2), T_(u->cat2, c2 + c1, 0), n, H / 2, W / 2, c2);
-  conv_mma<3, bf16>(T_(u->cat2, c2 + c1), L[10].wn, B(10), T_(u->d2a, c1), n, H / 2, W / 2, c2 + c1, c1, 1, s, u->err);
-  conv_mma<3, bf16>(T_(u->d2a, c1), L[11].wn, B(11), T_(u->d2b, c1), n, H / 2, W / 2, c1, c1, 1, s, u->err);
+  conv_tc<3, bf16>(T_(u->cat2, c2 + c1), L[10].c.wp, B(10), T_(u->d2a, c1), n, H / 2, W / 2, c2 + c1, c1, 1, u->err, s);
+  conv_tc<3, bf16>(T_(u->d2a, c1), L[11].c.wp, B(11), T_(u->d2b, c1), n, H / 2, W / 2, c1, c1, 1, u->err, s);
   k_up<<<grid((long long)n * H * W * c1 / 8), 256, 0, s>>>(T_(u->d2b, c1), T_(u->cat1, c1 + c0, 0), n, H, W, c1);
-  conv_mma<3, bf16>(T_(u->cat1, c1 + c0), L[12].wn, B(12), T_(u->d1a, c0), n, H, W, c1 + c0, c0, 1, s, u->err);
-  conv_mma<3, bf16>(T_(u->d1a, c0), L[13].wn, B(13), T_(u->d1b, c0), n, H, W, c0, c0, 1, s, u->err);
-  if (!conv_tc<1, float>(T_(u->d1b, c0), L[14].wn, B(14), none, n, H, W, c0, u->cout, 0, u->err, s, 1,
+  conv_tc<3, bf16>(T_(u->cat1, c1 + c0), L[12].c.wp, B(12), T_(u->d1a, c0), n, H, W, c1 + c0, c0, 1, u->err, s);
+  conv_tc<3, bf16>(T_(u->d1a, c0), L[13].c.wp, B(13), T_(u->d1b, c0), n, H, W, c0, c0, 1, u->err, s);
+  if (!conv_tc<1, float>(T_(u->d1b, c0), L[14].c.wp, B(14), none, n, H, W, c0, u->cout, 0, u->err, s, 1,
                          none, head)) {
     // a head wider than the tcgen05 tiles: pixel-major, then to its planar place
     const long long P = (long long)H * W;
-    conv_mma<1, float>(T_(u->d1b, c0), L[14].wn, B(14), T_(u->ynhwc, u->cout), n, H, W, c0, u->cout,
+    conv_mma<1, float>(T_(u->d1b, c0), L[14].c.wn, B(14), T_(u->ynhwc, u->cout), n, H, W, c0, u->cout,
                        0, s);
     k_unpack_out<<<grid1d(P * n), 256, 0, s>>>(u->ynhwc, head, P, u->cout, n);
     count_launches(1);
@@ -1314,9 +1433,9 @@ void layer_backward(ashrt_unet* u, Tensor in, const bf16* gz, const Layer& l, Te
   }
   const Tensor g = T_(const_cast<bf16*>(gz), l.co);
   if (gz_out)
-    conv_tc<3, bf16>(g, l.wtn, nullptr, T_(gz_out, l.ci), n, H, W, l.co, l.ci, 0, u->err, s, 0, act);
+    conv_tc<3, bf16>(g, l.c.wtp, nullptr, T_(gz_out, l.ci), n, H, W, l.co, l.ci, 0, u->err, s, 0, act);
   else
-    conv_tc<3, float>(g, l.wtn, nullptr, out, n, H, W, l.co, l.ci, 0, u->err, s);
+    conv_tc<3, float>(g, l.c.wtp, nullptr, out, n, H, W, l.co, l.ci, 0, u->err, s);
 }
 
 // Backward pass from the planar head output u->y and the targets; accumulates
@@ -1330,8 +1449,14 @@ void net_backward(ashrt_unet* u, const float* target, int n, cudaStream_t s) {
   const long long P = (long long)H * W;
   const dim3 hg((unsigned)std::min<long long>((P * n + kHeadPix - 1) / kHeadPix, 152 * 8),
                 (u->cout + kHeadCh - 1) / kHeadCh);
-  k_head_bwd<<<hg, kHeadPix, 0, s>>>(u->y, target, u->lam, u->d1b, L[14].wt, ga,
-                                     u->g + L[14].w_off, u->g + L[14].b_off, P, u->cout, n, u->loss);
+  const bool ws = u->cout <= kHeadMaxShared;
+  const size_t hs = ws ? u->cout * 16 * sizeof(float) : 0;
+  auto* head = ws ? k_head_bwd<true> : k_head_bwd<false>;
+  if (hs > 16 * 1024)
+    cudaFuncSetAttribute(head, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(kHeadMaxShared * 16 * sizeof(float)));
+  head<<<hg, kHeadPix, hs, s>>>(u->y, target, u->lam, u->d1b, L[14].c.wt, ga,
+                                u->g + L[14].w_off, u->g + L[14].b_off, P, u->cout, n, u->loss);
   // dec1
   layer_backward(u, T_(u->d1a, c0), ga, L[13], none, T_(u->d1a, c0), gb, n, H, W, s);
   layer_backward(u, T_(u->cat1, c1 + c0), gb, L[12], T_(u->gcat1, c1 + c0), none, nullptr, n, H, W, s);
@@ -1376,8 +1501,7 @@ void net_backward(ashrt_unet* u, const float* target, int n, cudaStream_t s) {
 cudaError_t refresh_bf16_weights(ashrt_unet* u, cudaStream_t s) {
   for (auto& l : u->L) {
     const int total = l.co * l.ci * l.k * l.k;
-    k_wconv<<<(total + 255) / 256, 256, 0, s>>>(u->w + l.w_off, l.wf, l.wt, l.wn, l.wtn, l.co,
-                                                l.ci, l.k);
+    k_wconv<<<(total + 255) / 256, 256, 0, s>>>(u->w + l.w_off, l.c, l.co, l.ci, l.k);
     count_launches(1);
   }
   return cudaGetLastError();
@@ -1427,10 +1551,23 @@ ashrt_status ashrt_unet_create(ashrt_unet** out, int H, int W, int out_channels,
   A(&u->am, off);
   A(&u->av, off);
   for (auto& l : u->L) {
-    A(&l.wf, (size_t)l.co * l.ci * l.k * l.k);
-    A(&l.wt, (size_t)l.co * l.ci * l.k * l.k);
-    A(&l.wn, (size_t)l.co * l.ci * l.k * l.k);
-    A(&l.wtn, (size_t)l.co * l.ci * l.k * l.k);
+    const size_t n = (size_t)l.co * l.ci * l.k * l.k;
+    const bool first = &l == &u->L.front();
+    if (first) A(&l.c.wf, n);
+    if (l.k == 1) {
+      A(&l.c.wt, n);
+      if (!tc_tile(1, l.co)) A(&l.c.wn, n);
+    }
+    if (!first && (l.c.nt_p = tc_tile(l.k, l.co))) {
+      // a head of any width fills whole tiles (zeros)
+      const size_t np = n / l.co * ((l.co + l.c.nt_p - 1) / l.c.nt_p * l.c.nt_p);
+      A(&l.c.wp, np);
+      if (e == cudaSuccess) e = cudaMemset(l.c.wp, 0, np * sizeof(bf16));
+    }
+    if (!first && l.k == 3) {
+      l.c.nt_t = tc_tile(3, l.ci);
+      A(&l.c.wtp, n);
+    }
   }
   A(&u->x, P0);
   A(&u->e1a, P0 * c0);
