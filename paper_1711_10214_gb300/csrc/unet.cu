@@ -1264,16 +1264,23 @@ void net_forward(ashrt_unet* u, int n, cudaStream_t s, const HeadOut& head) {
 // is copied once and no copy is waited for.  Both operands stay in their NHWC
 // order and are read with ldmatrix.trans (row pitches of an odd number of 16-byte
 // units: no bank conflicts); a tap that looks across the image's first or last
-// row is left out for that row.  The FP32 partial sums leave with one atomic
-// each; CTAs of the first input-channel tile also sum the bias gradient.
+// row is left out for that row.  The
+// tensor core's FP32 accumulation truncates, so its error grows with the length of a
+// chain (584 steps of 16 pixels left 1.7e-5 of a gradient's norm, 216 a third of
+// it): after `chain` rows a sum moves on, to a second set of registers where a tile
+// has them to spare, with an atomic each otherwise.  CTAs of the first
+// input-channel tile also sum the bias gradient.
 // Channel tiles of 48 x 48 (the network's channels are multiples of 48 but for
 // 16 and 64) waste nothing where 32 x 32 computed a third to a half of padding.
+// 8 images 256 x 1024, all thirteen layers: 2.86 ms with a wait per row and no
+// ring, 1.69 ms so, of which the shorter chains take 0.24.
 struct WgMmaArgs {
   Tensor in;            // bf16 layer input slice (ps, off multiples of 8)
   const bf16* gz;       // bf16 masked output gradient, dense [pixels][Cout]
   float* gw;            // [Cout][Cin][3][3] fp32, accumulated
   float* gb;            // [Cout] fp32, accumulated
   int N, H, W, Cin, Cout, rows_per;
+  int chain;            // image rows summed in one chain of the tensor core's accumulators
 };
 
 __device__ __forceinline__ void ldsm_x4_t(uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3,
@@ -1331,6 +1338,28 @@ __global__ void __launch_bounds__(288, MT * NT >= 18 ? 2 : 3) k_wgrad_mma(WgMmaA
     for (int j = 0; j < NT; ++j) acc[i][j][0] = acc[i][j][1] = acc[i][j][2] = acc[i][j][3] = 0.f;
   float bsum = 0.f;
   const bool bias = blockIdx.y == 0 && tid < PARTS * CO_T;
+  constexpr bool TWO = MT * NT <= 6;            // registers for the sums of several chains
+  float sum[MT][NT][4];   // (unused and so without registers otherwise)
+  if (TWO) {
+#pragma unroll
+    for (int i = 0; i < MT; ++i)
+#pragma unroll
+      for (int j = 0; j < NT; ++j) sum[i][j][0] = sum[i][j][1] = sum[i][j][2] = sum[i][j][3] = 0.f;
+  }
+  auto to_memory = [&](const float (&v)[MT][NT][4]) {
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int i = 0; i < MT; ++i)
+#pragma unroll
+      for (int j = 0; j < NT; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int co = co0 + i * 16 + g + 8 * (e >> 1), ci = ci0 + j * 8 + 2 * t + (e & 1);
+          if (co < a.Cout && ci < a.Cin)
+            atomicAdd(&a.gw[((long long)co * a.Cin + ci) * 9 + tap], v[i][j][e]);
+        }
+  };
+  int left = a.chain;
 
   load_x(row0 - 1);
   load_x(row0);
@@ -1349,6 +1378,19 @@ __global__ void __launch_bounds__(288, MT * NT >= 18 ? 2 : 3) k_wgrad_mma(WgMmaA
     if (bias)
       for (int px = tid / CO_T; px < 128; px += PARTS)
         bsum += __bfloat162float(g[px * LDG + tid % CO_T]);
+    if (left-- == 0) {   // the chain ends: its sum moves on, rounded to nearest
+      left = a.chain - 1;
+      if (!TWO) to_memory(acc);
+#pragma unroll
+      for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            if (TWO) sum[i][j][e] += acc[i][j][e];
+            acc[i][j][e] = 0.f;
+          }
+    }
     const int y = row % a.H;
     if ((dy == 0 && y == 0) || (dy == 2 && y == a.H - 1)) continue;
     const bf16* x = xs + ((row + dy - 1) & 3) * PW * LDX + dx * LDX;
@@ -1372,17 +1414,15 @@ __global__ void __launch_bounds__(288, MT * NT >= 18 ? 2 : 3) k_wgrad_mma(WgMmaA
       }
     }
   }
-  const int g = lane >> 2, t = lane & 3;
+  if (TWO) {
 #pragma unroll
-  for (int i = 0; i < MT; ++i)
+    for (int i = 0; i < MT; ++i)
 #pragma unroll
-    for (int j = 0; j < NT; ++j)
+      for (int j = 0; j < NT; ++j)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int co = co0 + i * 16 + g + 8 * (e >> 1), ci = ci0 + j * 8 + 2 * t + (e & 1);
-        if (co < a.Cout && ci < a.Cin)
-          atomicAdd(&a.gw[((long long)co * a.Cin + ci) * 9 + tap], acc[i][j][e]);
-      }
+        for (int e = 0; e < 4; ++e) acc[i][j][e] += sum[i][j][e];
+  }
+  to_memory(acc);
   if (bias && co0 + tid % CO_T < a.Cout) atomicAdd(&a.gb[co0 + tid % CO_T], bsum);
 }
 
@@ -1402,6 +1442,11 @@ void wgrad_mma_v(const WgMmaArgs& a0, cudaStream_t s) {
   const long long rows = (long long)a.N * a.H, want = 152LL * res / ((long long)gy * gz * xt);
   const long long per_col = std::max(1LL, std::min(want, rows));
   a.rows_per = (int)((rows + per_col - 1) / per_col);
+  // rows to a chain: as many as give about 152 x 8 chains in all per 32 x 32 channels
+  // (32 x 16 for 16 output channels)
+  const long long tiles = (long long)((a.Cin + 31) / 32) * (a.Cout <= 16 ? 1 : (a.Cout + 31) / 32);
+  const long long chains = std::min(rows, ((152LL * 8 + tiles - 1) / tiles + xt - 1) / xt);
+  a.chain = (int)((rows + chains - 1) / chains);
   const long long nstrip = (rows + a.rows_per - 1) / a.rows_per;
   k_wgrad_mma<MT, NT><<<dim3((unsigned)(nstrip * xt), gy, gz), 288, smem, s>>>(a);
   count_launches(1);
