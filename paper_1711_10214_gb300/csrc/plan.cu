@@ -181,16 +181,17 @@ size_t data_elems(const ashrt_plan* p) { return (size_t)p->nr * p->nt; }
 //     against 4790 / 5258.
 //   Nt 1024: the single-gather form: 16 panels, 129 rows, 16 gathers 95 / 94
 //     against 121 / 111 (4), 64 gathers 347 / 338 against 336 / 369.
-//   Nt 2048, 32 panels, 257 rows: the pair form (9) shares each twiddle and
-//     table read between two gathers, which wins once pairs alone fill the
-//     chip: forward 3 gathers (R = 771) 158 single against 175, 4 (1028) 191
-//     against 179; adjoint 12 gathers (3084) 511 against 518, 64 gathers 2593
-//     against 2491.  So single below R = 900 (forward) and 3600 (adjoint).
+//   Nt 2048, 32 panels, 257 rows: the pair form (9) shares each tap and
+//     table read between two gathers, which wins once pairs alone nearly fill the
+//     chip: forward 1 gather (R = 257) 64 single against 102, 2 (514) 110 against
+//     102, 4 (1028) 191 against 153; adjoint 12 gathers (3084) 511 against 518, 64
+//     gathers 2593 against 2491.  So single below R = 400 (forward) and 3600
+//     (adjoint).
 int rows_variant(const ashrt_plan* p, int batch) {
   if (p->rows_minb) return p->rows_minb;
   if (p->logNt != 11) return 6;
   const long long R = (long long)batch * p->Lh;
-  return R <= 900 ? 6 : (R <= 3600 ? 10 : 9);
+  return R <= 400 ? 6 : (R <= 3600 ? 10 : 9);
 }
 
 // ---------------------------------------------------------------------------

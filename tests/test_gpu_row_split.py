@@ -50,7 +50,7 @@ def test_split_panels_match_oracle(lib, nt, nx, nv, t0, batch):
 
 
 @pytest.mark.parametrize("nt,nx,nv,nt0,batch,fixed", [
-    (600, 60, 6, 1, 8, 9),       # Nt 2048, 520 rows: single-gather both
+    (600, 60, 6, 1, 8, 9),       # Nt 2048, 520 rows
     (1000, 100, 6, 1, 7, 9),     # 903 rows: tensor-memory forward, single-gather adjoint
     (1000, 100, 4, 2, 16, 6),    # the same, shifts
     (1000, 250, 3, 1, 15, 9),    # 3855 rows: the pair form both ways
