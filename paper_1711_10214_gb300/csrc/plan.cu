@@ -181,17 +181,16 @@ size_t data_elems(const ashrt_plan* p) { return (size_t)p->nr * p->nt; }
 //     against 4790 / 5258.
 //   Nt 1024: the single-gather form: 16 panels, 129 rows, 16 gathers 95 / 94
 //     against 121 / 111 (4), 64 gathers 347 / 338 against 336 / 369.
-//   Nt 2048, 32 panels, 257 rows: the pair form (9) shares each tap and
-//     table read between two gathers, which wins once pairs alone nearly fill the
-//     chip: forward 1 gather (R = 257) 64 single against 102, 2 (514) 110 against
-//     102, 4 (1028) 191 against 153; adjoint 12 gathers (3084) 511 against 518, 64
-//     gathers 2593 against 2491.  So single below R = 400 (forward) and 3600
-//     (adjoint).
+//   Nt 2048: the pair form's forward (9) from two gathers on: 32 panels, 129 rows:
+//     1 gather 37 single against 53, 2 gathers 65 against 52; 257 rows: 2 gathers 110
+//     against 88, 3 164 against 151, 4 192 against 152; 192 panels, 129 rows, 2
+//     gathers 350 against 224.  The adjoint's pair form shares each twiddle and
+//     table read between two gathers, which wins once pairs alone fill the chip:
+//     12 gathers (R = 3084) 511 against 518, 64 gathers 2593 against 2491.
 int rows_variant(const ashrt_plan* p, int batch) {
   if (p->rows_minb) return p->rows_minb;
-  if (p->logNt != 11) return 6;
-  const long long R = (long long)batch * p->Lh;
-  return R <= 400 ? 6 : (R <= 3600 ? 10 : 9);
+  if (p->logNt != 11 || batch < 2) return 6;
+  return (long long)batch * p->Lh <= 3600 ? 10 : 9;
 }
 
 // ---------------------------------------------------------------------------

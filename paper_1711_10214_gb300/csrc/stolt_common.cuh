@@ -234,7 +234,8 @@ __device__ __forceinline__ void panel_chunk(int P, int n, int z, int& p0, int& p
 // 256 x 64, 8 panels (65 rows) 16.3 / 18.2 -> 11.0 / 10.4 us; 2 gathers
 // 181 x 455, 25 panels (513 rows of pairs) 51 / 54 -> 45 / 41 us; 1 gather
 // 1024 x 256, 32 panels (257 rows, single-gather form) 75 / 82 -> 62 / 60 us;
-// 2 gathers 1024 x 128, 192 panels (258 rows) 451 / 555 -> 349 / 347 us.
+// 2 gathers 1024 x 128, 192 panels (258 rows) 451 / 555 -> 349 / 347 us, as 129
+// pairs 459 -> 224 us forward.
 inline int rows_split(long long ctas, int P, int res, bool ordered) {
   constexpr int kSms = 152;
   int best = 1;

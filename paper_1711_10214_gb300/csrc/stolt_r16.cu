@@ -521,7 +521,8 @@ __global__ void __launch_bounds__(128, 4) stolt_fwd_rows16_tm(RowArgs a) {
 // issue of instructions then, so sums of complex numbers are packed (f32x2) and the
 // map is pared down (400 M warp instructions, 518 M plain).  The sums and the
 // twiddles lie in tensor memory as there.  16 gathers: 610 -> 500 us; 64: 2280 ->
-// 1860 us (input read once at the measured copy rate: 320 us).
+// 1860 us (input read once at the measured copy rate: 320 us).  Few rows are split
+// by panels (rows_split): 2 gathers 1024 x 128, 192 panels 459 -> 224 us.
 // roots of unity exp(-2 pi i m / 64)
 struct Roots64 {
   float c[64], s[64];
@@ -634,7 +635,8 @@ __device__ __forceinline__ float2 root2048(const float2* __restrict__ tw, int m)
 
 constexpr int kSide32 = 32 * 33;   // a warp's 32 x 32 exchange, rows padded by one
 
-template <bool SHIFT>
+// SPLIT: the panels are split over the CTAs of a cluster along the grid's z.
+template <bool SHIFT, bool SPLIT>
 __global__ void __launch_bounds__(128, 4) stolt_fwd_rows32_tm(RowArgs a) {
   constexpr int LOGN = 11, N = 1 << LOGN, T = 128, H = N / 2;
   using S = Sched16<LOGN>;
@@ -679,8 +681,10 @@ __global__ void __launch_bounds__(128, 4) stolt_fwd_rows32_tm(RowArgs a) {
     tm_wait_st();
   }
 
-  int iv = 0, jt = 0;
-  for (int p = 0; p < a.P; ++p) {
+  int p0 = 0, p1 = a.P;
+  if (SPLIT) panel_chunk(a.P, a.psplit, blockIdx.z, p0, p1);
+  int iv = SPLIT ? p0 % a.nv : 0, jt = SPLIT ? p0 / a.nv : 0;
+  for (int p = p0; p < p1; ++p) {
     const float2* xp = x + (long long)p * a.x_panel;
     float2 v[32];
 #pragma unroll
@@ -697,7 +701,7 @@ __global__ void __launch_bounds__(128, 4) stolt_fwd_rows32_tm(RowArgs a) {
     __syncthreads();                            // every read of the previous panel's map is done
     stage_taps(stap, trow + iv * tstep, a.taps_ld, tid, T);
     cp_async_commit();
-    if (p + 1 < a.P && (tid & 63) * 16 < a.nt)
+    if (p + 1 < p1 && (tid & 63) * 16 < a.nt)
       asm volatile("prefetch.global.L2 [%0];\n" ::"l"(xp + a.x_panel + (tid & 63) * 16));
     if (odd) {
       constexpr Roots64 w;
@@ -733,7 +737,7 @@ __global__ void __launch_bounds__(128, 4) stolt_fwd_rows32_tm(RowArgs a) {
       uint32_t r[16];
       tm_ld16(tacc + 16 * c, r);
       tm_wait_ld(r);
-      if (SHIFT && iv == 0 && p > 0) {
+      if (SHIFT && iv == 0 && p > p0) {
         // shift jt - 1 -> jt: the sums move to the new shift's phase frame
         const float2* ph1 = a.phase + (long long)jt * N;
         const float2* ph0 = ph1 - N;
@@ -795,14 +799,14 @@ __global__ void __launch_bounds__(128, 4) stolt_fwd_rows32_tm(RowArgs a) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(*tslot),
                  "r"((uint32_t)(2 * kTmCols)));
   }
-  // with asymptote shifts the sums are in the last shift's phase frame
-  const float2* phl = SHIFT ? a.phase + (long long)(a.nt0 - 1) * N : nullptr;
+  if (SHIFT && p0 < p1) {   // the sums are in the phase frame of the last panel's shift
+    const float2* phl = a.phase + (long long)((p1 - 1) / a.nv) * N;
 #pragma unroll
-  for (int s = 0; s < 16; ++s) {
-    const int k = tid + T * s;
-    if (SHIFT) acc[s] = cmul(acc[s], __ldg(phl + k));
-    acc[s] = cscale(acc[s], __ldg(a.wt + k));
+    for (int s = 0; s < 16; ++s) acc[s] = cmul(acc[s], __ldg(phl + tid + T * s));
   }
+  if (SPLIT && !cluster_sum_rows<16, T>(buf, acc, tid, a.psplit)) return;
+#pragma unroll
+  for (int s = 0; s < 16; ++s) acc[s] = cscale(acc[s], __ldg(a.wt + tid + T * s));
   r16_first_pass<+1>(buf, acc, tid);
   r16_pass_range<+1, LOGN, 1, S::NPASS - 1>(buf, a.tw16, tid);
   float2* yA = a.Yw + (long long)b0 * a.y_batch + (long long)l * a.ld;
@@ -823,14 +827,17 @@ cudaError_t launch_fwd16_tm(const RowArgs& a, cudaStream_t s) {
 }
 
 template <bool SHIFT>
-cudaError_t launch_fwd32_tm(const RowArgs& a, cudaStream_t s) {
+cudaError_t launch_fwd32_tm(const RowArgs& a0, cudaStream_t s) {
   constexpr int N = 1 << 11;
-  static bool attr = false;
+  RowArgs a = a0;
+  const dim3 grid(a.Lh, (a.batch + 1) / 2);
+  a.psplit = rows_split((long long)grid.x * grid.y, a.P, 4, true);
   static_assert(4 * kSide32 * sizeof(float2) >= N * sizeof(float4), "the final transform's row");
   const size_t smem = 4 * kSide32 * sizeof(float2) + (size_t)a.taps_ld * sizeof(unsigned) + 16;
-  cudaError_t e = set_smem(stolt_fwd_rows32_tm<SHIFT>, smem_cap<11>(true), attr);
-  if (e != cudaSuccess) return e;
-  stolt_fwd_rows32_tm<SHIFT><<<dim3(a.Lh, (a.batch + 1) / 2), 128, smem, s>>>(a);
+  if (a.psplit > 1)
+    return launch_cluster_z(stolt_fwd_rows32_tm<SHIFT, true>, dim3(grid.x, grid.y, a.psplit), 128,
+                            smem, a.psplit, s, a);
+  stolt_fwd_rows32_tm<SHIFT, false><<<grid, 128, smem, s>>>(a);
   return cudaGetLastError();
 }
 

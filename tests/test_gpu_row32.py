@@ -17,6 +17,7 @@ DT, DX = 0.004, 12.5
     (1023, 9, 2, None, 3, 2),                 # a group of rows short by one, an odd batch
     (513, 4, 1, None, 1, 2),                  # the shortest rows, one panel, no second gather
     (769, 12, 3, [0.0, 0.02, 0.05], 5, 2),    # a group's first sample only, shifts
+    (600, 16, 3, [0.0, 0.02, 0.05], 2, 2),    # 9 panels in 8 chunks that begin inside a shift
     (1025, 6, 2, None, 2, 1),                 # longer than Nt / 2: the 16 x 16 x 8 form
     (2048, 5, 2, [0.0, 0.03], 3, 1),
 ])
