@@ -15,11 +15,16 @@
 // on the host in FP64 (c_l folded into the synthesis table).
 //
 // Both are dense complex contractions per gather, M x N x K = nr x nt x Lh
-// and Lh x nt x nr, done here as FP32 tiled kernels on the CUDA cores: a
-// 64 x 64 output tile per CTA, K staged through shared memory in chunks of
-// 16, 4 x 4 outputs per thread.  The IRLS weights and the trace mask are
-// fused into the synthesis epilogue (with the per-gather squared norm of the
-// output for the CG scalars) and into the analysis operand load.
+// and Lh x nt x nr, done here as FP32 tiled kernels on the CUDA cores, bound by
+// their FP32 multiply-adds: 128 samples by 64 traces (32 wavenumbers) per CTA of
+// 128 threads, 64 accumulators per thread in an outer product (each value read
+// from shared memory serves 8 or 16 multiply-adds; with 16 accumulators the shared
+// memory pipe was the bound), K in double-buffered chunks of eight with one barrier
+// each.  The IRLS weights and the trace mask are fused into the synthesis epilogue
+// (with the per-gather squared norm of the output for the CG scalars) and into the
+// analysis operand load.  A sum runs over K in ascending order as before.
+// 16 gathers 1024 x 256, 257 wavenumbers: 212 -> 123 us (35 TFLOP/s) and 162 ->
+// 131 us (the 257th wavenumber's tile row included).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -30,7 +35,28 @@
 namespace ashrt {
 namespace {
 
-constexpr int kBM = 64, kBN = 64, kBK = 16, kThr = 256;
+constexpr int kThr = 128, kBN = 128, kBK = 8;
+constexpr int kSynM = 64, kAnaM = 32;   // traces (synthesis), wavenumbers (analysis) per CTA
+
+// n bytes from src, the rest of the 16, 8 or 4 zero
+__device__ __forceinline__ void cp_zfill16(void* dst, const void* src, int n) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(n)
+               : "memory");
+}
+__device__ __forceinline__ void cp_zfill8(void* dst, const void* src, int n) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(n)
+               : "memory");
+}
+__device__ __forceinline__ void cp_zfill4(void* dst, const void* src, int n) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(n)
+               : "memory");
+}
 
 __device__ __forceinline__ double warp_sum_dbl(double x) {
 #pragma unroll
@@ -39,82 +65,88 @@ __device__ __forceinline__ double warp_sum_dbl(double x) {
 }
 
 // d[g][j][t] = (sum_l Re(Es[j][l] Y[g][l][t])) * ew[g][j][t] * tmask[g][j];
-// dot[g] += sum d^2.  grid (ceil(nt/64), ceil(nr/64), batch).
-__global__ void __launch_bounds__(kThr) k_irr_synth(const float2* __restrict__ Es,
-                                                    const float2* __restrict__ Y,
-                                                    float* __restrict__ d, int nr, int nt, int Lh,
-                                                    int ld, long long y_batch,
-                                                    const float* __restrict__ ew,
-                                                    const float* __restrict__ tmask,
-                                                    double* __restrict__ dot) {
-  __shared__ float2 As[kBK][kBM];   // As[l][j]
-  __shared__ float2 Bs[kBK][kBN];   // Bs[l][t]
+// dot[g] += sum d^2.  grid (ceil(nt/128), ceil(nr/64), batch).  Rows of Y are
+// 16-byte aligned (ld a multiple of 4).
+__global__ void __launch_bounds__(kThr, 4) k_irr_synth(const float2* __restrict__ Es,
+                                                       const float2* __restrict__ Y,
+                                                       float* __restrict__ d, int nr, int nt, int Lh,
+                                                       int ld, long long y_batch,
+                                                       const float* __restrict__ ew,
+                                                       const float* __restrict__ tmask,
+                                                       double* __restrict__ dot) {
+  __shared__ __align__(16) float2 As[2][kBK][kSynM + 2];   // [l][j]
+  __shared__ __align__(16) float2 Bs[2][kBK][kBN];         // [l][t]
+  // thread: traces ty 8 .. + 7, samples 2 tx + 32 q + {0, 1}
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int t0 = blockIdx.x * kBN, j0 = blockIdx.y * kBM, g = blockIdx.z;
+  const int t0 = blockIdx.x * kBN, j0 = blockIdx.y * kSynM, g = blockIdx.z;
   const float2* Yg = Y + (long long)g * y_batch;
-  float acc[4][4];
+  auto load = [&](int k0, int buf) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[i][q] = 0.f;
-  for (int k0 = 0; k0 < Lh; k0 += kBK) {
-    // A chunk: 64 j x 16 l complex; thread loads 4 (one j, 4 consecutive l)
-    {
-      const int jj = tid >> 2, kk = (tid & 3) * 4;
-      const int j = j0 + jj;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int l = k0 + kk + u;
-        As[kk + u][jj] = (j < nr && l < Lh) ? __ldg(Es + (long long)j * Lh + l)
-                                            : make_float2(0.f, 0.f);
-      }
+    for (int u = 0; u < 4; ++u) {              // eight l of a trace in adjacent threads
+      const int kk = tid & 7, jj = (tid >> 3) + 16 * u, l = k0 + kk, j = j0 + jj;
+      const bool in = j < nr && l < Lh;
+      cp_zfill8(&As[buf][kk][jj], in ? Es + (long long)j * Lh + l : Es, in ? 8 : 0);
     }
-    // B chunk: 16 l x 64 t complex; thread loads 4 consecutive t of one l
-    {
-      const int kk = tid >> 4, tt = (tid & 15) * 4;
-      const int l = k0 + kk;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int t = t0 + tt + u;
-        Bs[kk][tt + u] = (l < Lh && t < nt) ? __ldg(Yg + (long long)l * ld + t)
-                                            : make_float2(0.f, 0.f);
-      }
+    for (int u = 0; u < 4; ++u) {              // two samples at a time, 64 threads a row
+      const int kk = (tid >> 6) + 2 * u, tt = 2 * (tid & 63), l = k0 + kk, t = t0 + tt;
+      const int n = l < Lh && t < nt ? (t + 1 < nt ? 16 : 8) : 0;
+      cp_zfill16(&Bs[buf][kk][tt], n ? Yg + (long long)l * ld + t : Yg, n);
     }
-    __syncthreads();
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  float acc[8][8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int q = 0; q < 8; ++q) acc[i][q] = 0.f;
+  load(0, 0);
+  for (int k0 = 0, buf = 0; k0 < Lh; k0 += kBK, buf ^= 1) {
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();   // this chunk is there; the other buffer's reads are done
+    if (k0 + kBK < Lh) load(k0 + kBK, buf ^ 1);
 #pragma unroll
     for (int k = 0; k < kBK; ++k) {
-      float2 a[4], b[4];
+      float4 a[4], b[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[k][ty * 4 + i];
+      for (int i = 0; i < 4; ++i) a[i] = *(const float4*)&As[buf][k][ty * 8 + 2 * i];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) b[q] = Bs[k][tx * 4 + q];
+      for (int q = 0; q < 4; ++q) b[q] = *(const float4*)&Bs[buf][k][2 * tx + 32 * q];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[i][q] = fmaf(a[i].x, b[q].x, fmaf(-a[i].y, b[q].y, acc[i][q]));
+        for (int q = 0; q < 4; ++q) {
+          float* c0 = &acc[2 * i][2 * q];
+          float* c1 = &acc[2 * i + 1][2 * q];
+          c0[0] = fmaf(a[i].x, b[q].x, fmaf(-a[i].y, b[q].y, c0[0]));
+          c0[1] = fmaf(a[i].x, b[q].z, fmaf(-a[i].y, b[q].w, c0[1]));
+          c1[0] = fmaf(a[i].z, b[q].x, fmaf(-a[i].w, b[q].y, c1[0]));
+          c1[1] = fmaf(a[i].z, b[q].z, fmaf(-a[i].w, b[q].w, c1[1]));
+        }
     }
-    __syncthreads();
   }
-  float part = 0.f;
+  double part = 0.0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int j = j0 + ty * 4 + i;
+  for (int i = 0; i < 8; ++i) {
+    const int j = j0 + ty * 8 + i;
     if (j >= nr) continue;
     const float tm = tmask ? __ldg(tmask + (long long)g * nr + j) : 1.f;
     const long long row = ((long long)g * nr + j) * nt;
+    float p = 0.f;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int t = t0 + tx * 4 + q;
+    for (int q = 0; q < 8; ++q) {
+      const int t = t0 + 2 * tx + 32 * (q >> 1) + (q & 1);
       if (t >= nt) continue;
       float v = acc[i][q] * tm;
       if (ew) v *= __ldg(ew + row + t);
       d[row + t] = v;
-      part = fmaf(v, v, part);
+      p = fmaf(v, v, p);
     }
+    part += (double)p;
   }
   if (dot) {
     __shared__ double red[kThr / 32];
-    double p = warp_sum_dbl((double)part);
+    double p = warp_sum_dbl(part);
     if ((tid & 31) == 0) red[tid >> 5] = p;
     __syncthreads();
     if (tid < 32) {
@@ -126,67 +158,82 @@ __global__ void __launch_bounds__(kThr) k_irr_synth(const float2* __restrict__ E
 }
 
 // Yhat[g][l][t] = sum_j Ea[l][j] (d[g][j][t] * ew[g][j][t] * tmask[g][j]),
-// Ea = conj(E)^T.  grid (ceil(nt/64), ceil(Lh/64), batch).
-__global__ void __launch_bounds__(kThr) k_irr_analysis(const float2* __restrict__ Ea,
-                                                       const float* __restrict__ d,
-                                                       float2* __restrict__ Yh, int nr, int nt,
-                                                       int Lh, int ld, long long y_batch,
-                                                       const float* __restrict__ ew,
-                                                       const float* __restrict__ tmask) {
-  __shared__ float2 As[kBK][kBM];   // As[j][l]
-  __shared__ float Bs[kBK][kBN];    // Bs[j][t]
+// Ea = conj(E)^T.  grid (ceil(nt/128), ceil(Lh/32), batch).  There is always one
+// wavenumber more than a multiple of 32 (Nx >= 64): a warp without any skips the
+// multiply-adds.
+__global__ void __launch_bounds__(kThr, 4) k_irr_analysis(const float2* __restrict__ Ea,
+                                                          const float* __restrict__ d,
+                                                          float2* __restrict__ Yh, int nr, int nt,
+                                                          int Lh, int ld, long long y_batch,
+                                                          const float* __restrict__ ew,
+                                                          const float* __restrict__ tmask) {
+  __shared__ __align__(16) float2 As[2][kBK][kAnaM + 2];   // [j][l]
+  __shared__ __align__(16) float Bs[2][kBK][kBN];          // [j][t]
+  __shared__ float Ws[2][kBK][kBN];                        // [j][t]: ew
+  // thread: wavenumbers 4 ty .. + 3, samples 4 tx + 64 h + 0 .. 3
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int t0 = blockIdx.x * kBN, l0 = blockIdx.y * kBM, g = blockIdx.z;
-  float2 acc[4][4];
+  const int t0 = blockIdx.x * kBN, l0 = blockIdx.y * kAnaM, g = blockIdx.z;
+  const bool work = l0 + 8 * (tid >> 5) < Lh;
+  // (copied past the registers: the compiler moves register loads down to their use)
+  float tmn = 1.f;                             // the mask of the trace that the thread copies
+  auto load = [&](int k0, int buf) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int ll = tid >> 2, kk = 2 * (tid & 3) + u, l = l0 + ll, j = k0 + kk;
+      const bool in = l < Lh && j < nr;
+      cp_zfill8(&As[buf][kk][ll], in ? Ea + (long long)l * nr + j : Ea, in ? 8 : 0);
+    }
+    const int j = k0 + ty;
+    if (tmask) tmn = j < nr ? __ldg(tmask + (long long)g * nr + j) : 1.f;
+    const long long row = ((long long)g * nr + j) * nt;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int t = t0 + tx + 16 * u;
+      const bool in = j < nr && t < nt;
+      cp_zfill4(&Bs[buf][ty][tx + 16 * u], in ? d + row + t : d, in ? 4 : 0);
+      if (ew) cp_zfill4(&Ws[buf][ty][tx + 16 * u], in ? ew + row + t : ew, in ? 4 : 0);
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  float2 acc[4][8];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) acc[i][q] = make_float2(0.f, 0.f);
-  for (int k0 = 0; k0 < nr; k0 += kBK) {
-    {
-      const int ll = tid >> 2, kk = (tid & 3) * 4;
-      const int l = l0 + ll;
+    for (int q = 0; q < 8; ++q) acc[i][q] = make_float2(0.f, 0.f);
+  load(0, 0);
+  for (int k0 = 0, buf = 0; k0 < nr; k0 += kBK, buf ^= 1) {
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    if (tmask || ew) {                         // the thread's own copies
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int j = k0 + kk + u;
-        As[kk + u][ll] = (l < Lh && j < nr) ? __ldg(Ea + (long long)l * nr + j)
-                                            : make_float2(0.f, 0.f);
+      for (int u = 0; u < 8; ++u) {
+        float& v = Bs[buf][ty][tx + 16 * u];
+        v *= tmn;
+        if (ew) v *= Ws[buf][ty][tx + 16 * u];
       }
     }
-    {
-      const int kk = tid >> 4, tt = (tid & 15) * 4;
-      const int j = k0 + kk;
-      const float tm = (j < nr && tmask) ? __ldg(tmask + (long long)g * nr + j) : 1.f;
-      const long long row = ((long long)g * nr + j) * nt;
+    __syncthreads();   // this chunk is there; the other buffer's reads are done
+    if (k0 + kBK < nr) load(k0 + kBK, buf ^ 1);
+    if (work) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int t = t0 + tt + u;
-        float v = 0.f;
-        if (j < nr && t < nt) {
-          v = __ldg(d + row + t) * tm;
-          if (ew) v *= __ldg(ew + row + t);
-        }
-        Bs[kk][tt + u] = v;
+      for (int k = 0; k < kBK; ++k) {
+        float4 a[2], b[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) a[i] = *(const float4*)&As[buf][k][ty * 4 + 2 * i];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) b[h] = *(const float4*)&Bs[buf][k][4 * tx + 64 * h];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const float4 bv = b[q >> 2];
+            const float v = (q & 3) == 0 ? bv.x : (q & 3) == 1 ? bv.y : (q & 3) == 2 ? bv.z : bv.w;
+            acc[2 * i][q].x = fmaf(a[i].x, v, acc[2 * i][q].x);
+            acc[2 * i][q].y = fmaf(a[i].y, v, acc[2 * i][q].y);
+            acc[2 * i + 1][q].x = fmaf(a[i].z, v, acc[2 * i + 1][q].x);
+            acc[2 * i + 1][q].y = fmaf(a[i].w, v, acc[2 * i + 1][q].y);
+          }
       }
     }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kBK; ++k) {
-      float2 a[4];
-      float b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[k][ty * 4 + i];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) b[q] = Bs[k][tx * 4 + q];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          acc[i][q].x = fmaf(a[i].x, b[q], acc[i][q].x);
-          acc[i][q].y = fmaf(a[i].y, b[q], acc[i][q].y);
-        }
-    }
-    __syncthreads();
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -194,8 +241,8 @@ __global__ void __launch_bounds__(kThr) k_irr_analysis(const float2* __restrict_
     if (l >= Lh) continue;
     float2* out = Yh + (long long)g * y_batch + (long long)l * ld;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int t = t0 + tx * 4 + q;
+    for (int q = 0; q < 8; ++q) {
+      const int t = t0 + 4 * tx + 64 * (q >> 2) + (q & 3);
       if (t < nt) out[t] = acc[i][q];
     }
   }
@@ -242,7 +289,7 @@ bool build_irregular_tables(const double* x, int nr, int Nx, double dx, float2* 
 cudaError_t launch_irr_synth(const float2* Es, const float2* Y, float* d, int nr, int nt, int Lh,
                              int ld, long long y_batch, const float* ew, const float* tmask,
                              double* dot, int batch, cudaStream_t s) {
-  dim3 grid((nt + kBN - 1) / kBN, (nr + kBM - 1) / kBM, batch);
+  dim3 grid((nt + kBN - 1) / kBN, (nr + kSynM - 1) / kSynM, batch);
   k_irr_synth<<<grid, kThr, 0, s>>>(Es, Y, d, nr, nt, Lh, ld, y_batch, ew, tmask, dot);
   return cudaGetLastError();
 }
@@ -250,7 +297,7 @@ cudaError_t launch_irr_synth(const float2* Es, const float2* Y, float* d, int nr
 cudaError_t launch_irr_analysis(const float2* Ea, const float* d, float2* Yh, int nr, int nt,
                                 int Lh, int ld, long long y_batch, const float* ew,
                                 const float* tmask, int batch, cudaStream_t s) {
-  dim3 grid((nt + kBN - 1) / kBN, (Lh + kBM - 1) / kBM, batch);
+  dim3 grid((nt + kBN - 1) / kBN, (Lh + kAnaM - 1) / kAnaM, batch);
   k_irr_analysis<<<grid, kThr, 0, s>>>(Ea, d, Yh, nr, nt, Lh, ld, y_batch, ew, tmask);
   return cudaGetLastError();
 }
