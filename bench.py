@@ -149,8 +149,8 @@ KERNEL_SOURCES = {
                        "stolt_common.cuh", "common.cuh"],
     "stolt_fwd_rows": ["stolt_r16.cu", "stolt_fwd.cu", "stolt_r16s.cu", "stolt_r16.cuh",
                        "stolt_common.cuh", "common.cuh"],
-    "xfft_r2c": ["xfft.cu", "tma.cu", "tma.cuh", "common.cuh"],
-    "xfft_c2r": ["xfft.cu", "common.cuh"],
+    "xfft_r2c": ["xfft.cu", "xfft_half.cu", "xfft_common.cuh", "tma.cu", "tma.cuh", "common.cuh"],
+    "xfft_c2r": ["xfft.cu", "xfft_common.cuh", "common.cuh"],
 }
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic.md")
 
