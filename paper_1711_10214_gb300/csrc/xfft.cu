@@ -333,6 +333,22 @@ xfft_c2r_kernel(XfftArgs a) {
     cp_async_commit();
   }
 
+  // The spectrum tile that a CTA of the next wave takes, on its way into L2 (with the
+  // weight tile's copies the loads at the start are too few to cover HBM's latency:
+  // 8 gathers 1500 x 455, 24 panels, weighted, 607 -> 563 us; 16 gathers 1024 x 256, 32
+  // panels 431 -> 407.  Without weights it gains nothing: 315 and 320.)
+  if constexpr (PF && LOGN >= 9) {
+    const unsigned nb = blockIdx.x + 152 * (1024 / T);
+    if (nb < gridDim.x) {
+      const TileAt nx = tile_at(nb, a.nt, 2 * C);
+      const float2* ni = a.in_cplx + nx.slab * a.slab_cplx + nx.t0;
+      for (int row = tid; row <= N / 2; row += T) {
+        prefetch_l2(ni + (long long)row * a.ld);
+        if (C == 16 && nx.t0 + 16 < a.nt) prefetch_l2(ni + (long long)row * a.ld + 16);
+      }
+    }
+  }
+
   // first pass (radix 8: butterfly jb takes rows jb + r N/8) on Z = A + i B,
   // A and B the Hermitian-extended spectra of columns ta, ta + 1.  Row
   // jb + r N/8 > N/2 mirrors row (N/8 - jb) + (7 - r) N/8, so the thread

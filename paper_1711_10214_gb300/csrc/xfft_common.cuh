@@ -16,12 +16,17 @@ struct TileAt {
   unsigned slab;
   int t0;
 };
-__device__ __forceinline__ TileAt tile_at(int nt, int cols) {
+__device__ __forceinline__ TileAt tile_at(unsigned block, int nt, int cols) {
   const unsigned n = (unsigned)(nt + cols - 1) / (unsigned)cols;
   TileAt at;
-  at.slab = blockIdx.x / n;
-  at.t0 = (int)(blockIdx.x % n) * cols;
+  at.slab = block / n;
+  at.t0 = (int)(block % n) * cols;
   return at;
+}
+__device__ __forceinline__ TileAt tile_at(int nt, int cols) { return tile_at(blockIdx.x, nt, cols); }
+
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p));
 }
 inline unsigned tile_grid(int slabs, int nt, int cols) {
   return (unsigned)slabs * (unsigned)((nt + cols - 1) / cols);
