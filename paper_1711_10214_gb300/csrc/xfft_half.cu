@@ -80,6 +80,25 @@ xfft_r2c_half(XfftArgs a) {
   const float* ew = a.ew ? a.ew + slab * a.slab_real : nullptr;
   const float* tm = a.tmask ? a.tmask + (slab / a.slabs_per_gather) * a.nx : nullptr;
 
+  // The update's rows are loaded four at a time, each group's loads behind the stores
+  // of the one before: all of the tile's rows are sent on their way into L2 first (8
+  // gathers 1500 x 455, 24 panels, 987 -> 813 us; the next wave's tile as well or
+  // instead: slower, its lines meet the stores of this one).
+  if constexpr (CG) {
+    const bool up = a.cg_mode == 1;
+    const float4 cf = a.cg_coef[slab / a.slabs_per_gather];
+    const bool two = up && a.cg_p2_read && cf.w != 0.f;
+    const bool urw = up && a.cg_u_rw && (cf.z != 0.f || two);
+    const long long o0 = slab * a.slab_real + at.t0;
+    for (int row = tid; row < a.nx; row += M * C / 16) {
+      const long long o = o0 + (long long)row * a.nt;
+      prefetch_l2(a.cg_io + o);
+      prefetch_l2(a.cg_s + o);
+      if (urw) prefetch_l2(a.cg_u + o);
+      if (two) prefetch_l2((a.cg_pout ? a.cg_pout : a.cg_io) + o);
+    }
+  }
+
   // first pass: butterfly jb = j + J q takes rows jb + r M / R1
   {
     float2 x[16];
@@ -222,8 +241,16 @@ cudaError_t r2c_half_v(const XfftArgs& a, cudaStream_t s) {
 
 }  // namespace
 
+// With the fused CGLS update from six waves of CTAs on: it has half the length-N
+// kernel's threads per column, so with few tiles its groups of loads are a longer
+// chain.  Both, us per launch (length-N, this): N 512, 18 / 90 / 900 / 1800 tiles 14 / 12 /
+// 39 / 83 against 22 / 16 / 48 / 87; N 1024, 60 / 1200 / 1800 / 3600 tiles 14 / 58 / 90 /
+// 227 against 23 / 67 / 95 / 178.
 bool xfft_half_applies(const XfftArgs& a) {
-  return 2 * a.nx <= a.Nx && a.Nx >= 256 && a.Nx <= 1024;
+  if (2 * a.nx > a.Nx || a.Nx < 256 || a.Nx > 1024) return false;
+  if (!a.cg_mode) return true;
+  const int c = a.Nx < 1024 && a.cols == 16 ? 16 : 8, res = 512 / (a.Nx * c / 32);
+  return tile_grid(a.slabs, a.nt, 2 * c) >= 6u * 152u * (unsigned)res;
 }
 
 cudaError_t launch_xfft_r2c_half(const XfftArgs& a, cudaStream_t s) {
