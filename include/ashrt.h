@@ -196,10 +196,9 @@ ashrt_status ashrt_forward_static(int nt, int nx, double dt, double dx,
  *                with nt0 = 1 (ASHRT); nv * nt0 <= 256
  *   m_dev        [batch][nt0][nv][nx][nt] model (read by forward, written by adjoint)
  *   d_dev        [batch][nx][nt] data (written by forward, read by adjoint)
- * Asynchronous on `stream`, one kernel launch, no allocation, no plan.  The
- * forward accumulates with shared-memory atomic adds, so its last bits
- * depend on scheduling.  Argument errors return ASHRT_EINVAL before any
- * CUDA call.
+ * Asynchronous on `stream`, one kernel launch, no allocation, no plan; no
+ * atomics, so the result does not depend on the scheduling.  Argument errors
+ * return ASHRT_EINVAL before any CUDA call.
  */
 ashrt_status ashrt_td_forward(int nt, int nx, double dt, double dx, const float* velocities,
                               int nv, const float* t0_shifts, int nt0, const float* m_dev,
