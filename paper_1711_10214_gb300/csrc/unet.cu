@@ -32,21 +32,6 @@ __device__ __forceinline__ void st_f<float>(float* p, long long i, float v) { p[
 template <>
 __device__ __forceinline__ void st_f<bf16>(bf16* p, long long i, float v) { p[i] = __float2bfloat16(v); }
 
-// sum of w e^2 to about 2^-45 in FP32 pairs: exact products (fma residuals) and
-// Knuth's two-sum; the FP64 units are so few that three FP64 operations per
-// element bound the kernels that used them.
-struct SumSq2 {
-  float s = 0.f, c = 0.f;
-  __device__ __forceinline__ void add(float w, float e) {
-    const float q = w * e, qe = fmaf(w, e, -q);
-    const float p = q * e, pe = fmaf(qe, e, fmaf(q, e, -p));
-    const float t = s + p, z = t - s;
-    c += ((s - (t - z)) + (p - z)) + pe;
-    s = t;
-  }
-  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-};
-
 struct Tensor {        // a channel slice of an NHWC buffer
   void* p = nullptr;
   int ps = 0;          // channels allocated per pixel
@@ -105,16 +90,19 @@ __global__ void k_pack_in(const float* d, const float* rms, bf16* x, long long p
     x[i] = __float2bfloat16(d[i] / rms[i / per]);
 }
 
-// sum of squares of every gather, many CTAs per gather (FP64 partials, one
-// atomic per CTA), then rms = sqrt(sum / per)
+// sum of squares of every gather, many CTAs per gather (FP64 throughout: a gather's
+// amplitudes may be anywhere in FP32's range, and their squares are not; one atomic
+// per CTA), then rms = sqrt(sum / per)
 __global__ void k_sumsq(const float* d, long long per, double* acc) {
   const int n = blockIdx.y;
-  SumSq2 s;
+  double s = 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < per;
-       i += (long long)gridDim.x * blockDim.x)
-    s.add(1.f, d[n * per + i]);
+       i += (long long)gridDim.x * blockDim.x) {
+    const double v = d[n * per + i];
+    s = fma(v, v, s);
+  }
   __shared__ double red[256];
-  red[threadIdx.x] = s.value();
+  red[threadIdx.x] = s;
   __syncthreads();
   for (int o = blockDim.x / 2; o > 0; o >>= 1) {
     if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
@@ -260,13 +248,15 @@ __global__ void __launch_bounds__(256) k_pool_bwd_gz(Tensor g, Tensor gpool, Ten
 //   loss += sum_c lam_c mean (y - t)^2,   gy = its derivative (FP32, not stored),
 //   gz[p][:] = BF16 of the masked input gradient sum_c gy[p][c] w[c][:] (a > 0),
 //   gw[c][:] += sum_p gy[p][c] a[p][:],   gb[c] += sum_p gy[p][c],
-// all in FP32.  A CTA takes tiles of 128 pixels (one per thread) and, along the
-// grid's y, 32 output channels for gw; the y = 0 CTAs also form gz.  gy and the
-// tile's inputs meet in shared memory, where each warp adds its 32 pixels to its
-// own copy of gw: lane (ci, half) owns channels half, half + 2, ..  What bounds it
-// is HBM (y, t and the 16-channel maps once): 8 images 256 x 1024, 25 channels,
-// separate loss, weight- and input-gradient kernels 458 + 382 + 198 us and a mask
-// pass, this one 267 (with the loss in FP64, three operations per element, 504).
+// all in FP32 but the loss, which is summed in FP64: its squares leave FP32's range from
+// differences of 1.8e19 on (and below 1e-19).  A CTA takes tiles of 128 pixels (one per
+// thread) and, along the grid's y, 32 output channels for gw; the y = 0 CTAs also form
+// gz.  gy and the tile's inputs meet in shared memory, where each warp adds its 32
+// pixels to its own copy of gw: lane (ci, half) owns channels half, half + 2, ..  What
+// bounds it is HBM (y, t and the 16-channel maps once) and the FP64 units (a conversion,
+// a product and a multiply-add per output): 8 images 256 x 1024, 25 channels, a whole
+// training step 4.93 ms with the loss in pairs of FP32, 5.05 ms so (5.16 ms with lam
+// converted for every output).
 // WS: the head's weights (FP32) are in shared memory; else (very many channels) read
 // from global memory.
 constexpr int kHeadPix = 128, kHeadCh = 32, kHeadMaxShared = 1024;
@@ -282,10 +272,13 @@ __global__ void __launch_bounds__(kHeadPix) k_head_bwd(const float* __restrict__
   __shared__ __align__(16) float gys[kHeadCh][LD];
   __shared__ __align__(16) float as[16][LD];
   __shared__ double red[kHeadPix / 32];
-  extern __shared__ __align__(16) float wsh[];   // the head's weights [C][16]
+  extern __shared__ __align__(16) float wsh[];   // the head's weights [C][16], then lam [C] in FP64
+  double* const lsh = (double*)(wsh + C * 16);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (WS)
     for (int i = tid; i < C * 16; i += kHeadPix) wsh[i] = __bfloat162float(w[i]);
+  if (WS)
+    for (int i = tid; i < C; i += kHeadPix) lsh[i] = lam[i];
   const int cb = blockIdx.y * kHeadCh, ci = lane & 15, half = lane >> 4;
   const bool first = blockIdx.y == 0;
   const double inv = 1.0 / ((double)P * N);
@@ -295,7 +288,7 @@ __global__ void __launch_bounds__(kHeadPix) k_head_bwd(const float* __restrict__
   for (int k = 0; k < kHeadCh / 2; ++k) acc[k] = 0.f;
   for (int i = tid; i < kHeadCh * LD; i += kHeadPix) ((float*)gys)[i] = 0.f;   // channels >= C
   __syncthreads();
-  SumSq2 loss2;
+  double s = 0.0;                                // the loss, FP64 as its squares may leave FP32
   const long long total = P * N;
   for (long long t0 = blockIdx.x * (long long)kHeadPix; t0 < total;
        t0 += (long long)gridDim.x * kHeadPix) {
@@ -333,7 +326,8 @@ __global__ void __launch_bounds__(kHeadPix) k_head_bwd(const float* __restrict__
         const float g = inv2 * l * e;
         if (c >= cb && c < cb + kHeadCh) gys[c - cb][tid] = g;
         if (first) {
-          loss2.add(l, e);
+          const double e64 = e;
+          s = fma((WS ? lsh[c] : (double)l) * e64, e64, s);
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             float4 wv;
@@ -397,7 +391,6 @@ __global__ void __launch_bounds__(kHeadPix) k_head_bwd(const float* __restrict__
     if (c < C) atomicAdd(j < 16 ? gw + c * 16 + j : gb + c, sum[i]);
   }
   if (!first) return;
-  double s = loss2.value();
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) red[warp] = s;
   __syncthreads();
@@ -1495,11 +1488,11 @@ void net_backward(ashrt_unet* u, const float* target, int n, cudaStream_t s) {
   const dim3 hg((unsigned)std::min<long long>((P * n + kHeadPix - 1) / kHeadPix, 152 * 8),
                 (u->cout + kHeadCh - 1) / kHeadCh);
   const bool ws = u->cout <= kHeadMaxShared;
-  const size_t hs = ws ? u->cout * 16 * sizeof(float) : 0;
+  const size_t head_ch = 16 * sizeof(float) + sizeof(double), hs = ws ? u->cout * head_ch : 0;
   auto* head = ws ? k_head_bwd<true> : k_head_bwd<false>;
   if (hs > 16 * 1024)
     cudaFuncSetAttribute(head, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(kHeadMaxShared * 16 * sizeof(float)));
+                         (int)(kHeadMaxShared * head_ch));
   head<<<hg, kHeadPix, hs, s>>>(u->y, target, u->lam, u->d1b, L[14].c.wt, ga,
                                 u->g + L[14].w_off, u->g + L[14].b_off, P, u->cout, n, u->loss);
   // dec1
