@@ -7,6 +7,7 @@
 #include <string>
 
 #include "ashrt.h"
+#include "smem_attr.h"
 
 namespace ashrt {
 

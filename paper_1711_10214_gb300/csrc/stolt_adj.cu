@@ -120,7 +120,7 @@ stolt_adj_rows(RowArgs a) {
 template <int LOGN, bool SHIFT, int MINB, bool HALF>
 cudaError_t launch_adj_vh(const RowArgs& a, cudaStream_t s) {
   constexpr int N = 1 << LOGN;
-  static bool attr = false;
+  static SmemAttr attr;
   const size_t smem = (size_t)2 * N * sizeof(float4) + (size_t)a.atab_ld * sizeof(uint2);
   cudaError_t e = set_smem(stolt_adj_rows<LOGN, SHIFT, MINB, HALF>, smem_cap<LOGN>(false), attr);
   if (e != cudaSuccess) return e;

@@ -182,15 +182,6 @@ __device__ __forceinline__ void load_pair(float4* v, const float2* __restrict__ 
   }
 }
 
-template <typename K>
-inline cudaError_t set_smem(K kern, size_t bytes, bool& done) {
-  if (done || bytes <= 48 * 1024) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)bytes);
-  if (e == cudaSuccess) done = true;
-  return e;
-}
-
 // Shared bytes of the adjoint's source-table row (atab_row_len entries)
 inline constexpr size_t adj_tab_bytes(int N) { return (size_t)(((N / 2 + 1) + 1) & ~1) * 8; }
 

@@ -148,7 +148,7 @@ cudaError_t launch_fwd_vh(const RowArgs& a0, cudaStream_t s) {
     // longer rows have single-gather kernels for batches this small
     a.psplit = rows_split((long long)grid.x * grid.y, a.P, 8, true);
     if (a.psplit > 1) {
-      static bool attr = false;
+      static SmemAttr attr;
       cudaError_t e = set_smem(stolt_fwd_rows<LOGN, SHIFT, MINB, HALF, true>, smem_cap<LOGN>(true),
                                attr);
       if (e != cudaSuccess) return e;
@@ -156,7 +156,7 @@ cudaError_t launch_fwd_vh(const RowArgs& a0, cudaStream_t s) {
                               dim3(grid.x, grid.y, a.psplit), N / 8, smem, a.psplit, s, a);
     }
   }
-  static bool attr = false;
+  static SmemAttr attr;
   cudaError_t e = set_smem(stolt_fwd_rows<LOGN, SHIFT, MINB, HALF, false>, smem_cap<LOGN>(true),
                            attr);
   if (e != cudaSuccess) return e;

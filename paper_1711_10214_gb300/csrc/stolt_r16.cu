@@ -817,7 +817,7 @@ __global__ void __launch_bounds__(128, 4) stolt_fwd_rows32_tm(RowArgs a) {
 template <bool SHIFT>
 cudaError_t launch_fwd16_tm(const RowArgs& a, cudaStream_t s) {
   constexpr int N = 1 << 11;
-  static bool attr = false;
+  static SmemAttr attr;
   const size_t smem = (size_t)N * sizeof(float4) + (size_t)2 * a.ld * sizeof(float2) +
                       (size_t)a.taps_ld * sizeof(unsigned) + 16;
   cudaError_t e = set_smem(stolt_fwd_rows16_tm<SHIFT>, smem_cap<11>(true), attr);
@@ -848,7 +848,7 @@ cudaError_t launch_fwd32_tm(const RowArgs& a0, cudaStream_t s) {
 template <int LOGN, bool SHIFT, bool HALF>
 cudaError_t launch_fwd16_h(const RowArgs& a, cudaStream_t s) {
   constexpr int N = 1 << LOGN;
-  static bool attr = false;
+  static SmemAttr attr;
   const size_t smem = (size_t)N * sizeof(float4) + (size_t)2 * a.ld * sizeof(float2) +
                       (size_t)2 * a.taps_ld * sizeof(unsigned);
   cudaError_t e = set_smem(stolt_fwd_rows16<LOGN, SHIFT, HALF>, smem_cap<LOGN>(true), attr);
@@ -866,7 +866,7 @@ cudaError_t launch_fwd16(const RowArgs& a, cudaStream_t s) {
 template <int LOGN, bool SHIFT, bool HALF>
 cudaError_t launch_adj16_h(const RowArgs& a, cudaStream_t s) {
   constexpr int N = 1 << LOGN;
-  static bool attr = false;
+  static SmemAttr attr;
   const size_t smem = (size_t)2 * N * sizeof(float4) + (size_t)a.atab_ld * sizeof(uint2) + 16;
   cudaError_t e = set_smem(stolt_adj_rows16<LOGN, SHIFT, HALF>, smem_cap<LOGN>(false) + 16, attr);
   if (e != cudaSuccess) return e;

@@ -240,13 +240,13 @@ cudaError_t launch_fwd16s_h(const RowArgs& a0, cudaStream_t s) {
   a.psplit = rows_split((long long)a.batch * a.Lh, a.P, r16s_minb_fwd<LOGN>(), true);
   const size_t smem = (size_t)(N + a.ld) * sizeof(float2), cap = (size_t)2 * N * sizeof(float2);
   if (a.psplit > 1) {
-    static bool attr = false;
+    static SmemAttr attr;
     cudaError_t e = set_smem(stolt_fwd_rows16s<LOGN, SHIFT, HALF, true>, cap, attr);
     if (e != cudaSuccess) return e;
     return launch_cluster_z(stolt_fwd_rows16s<LOGN, SHIFT, HALF, true>,
                             dim3(a.batch, a.Lh, a.psplit), N / 16, smem, a.psplit, s, a);
   }
-  static bool attr = false;
+  static SmemAttr attr;
   cudaError_t e = set_smem(stolt_fwd_rows16s<LOGN, SHIFT, HALF, false>, cap, attr);
   if (e != cudaSuccess) return e;
   stolt_fwd_rows16s<LOGN, SHIFT, HALF, false><<<dim3(a.batch, a.Lh), N / 16, smem, s>>>(a);
@@ -262,7 +262,7 @@ cudaError_t launch_fwd16s(const RowArgs& a, cudaStream_t s) {
 template <int LOGN, bool SHIFT, bool HALF>
 cudaError_t launch_adj16s_h(const RowArgs& a, cudaStream_t s) {
   constexpr int N = 1 << LOGN;
-  static bool attr = false;
+  static SmemAttr attr;
   const size_t smem = (size_t)2 * N * sizeof(float2);
   cudaError_t e = set_smem(stolt_adj_rows16s<LOGN, SHIFT, HALF>, smem, attr);
   if (e != cudaSuccess) return e;

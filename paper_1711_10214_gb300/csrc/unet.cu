@@ -1075,12 +1075,8 @@ void conv_tc_v(const TcConvArgs& a, cudaStream_t s) {
   using S = TcTile<K, NT, RR>;
   const int nch = a.Cin / 16;
   const size_t smem = S::smem(nch);
-  static size_t attr = 0;
-  if (smem > attr) {
-    cudaFuncSetAttribute(k_conv_tc<K, NT, RR, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    attr = smem;
-  }
+  static SmemAttr attr;
+  set_smem(k_conv_tc<K, NT, RR, TO>, smem, attr);
   const int tiles = a.N * ((a.H + RR - 1) / RR) * ((a.W + 127) / 128);
   const int gy = (a.Cout + NT - 1) / NT;
   const int gx = std::min(tiles, std::max(1, 152 / gy));   // one CTA per SM
@@ -1137,12 +1133,8 @@ template <int K, int KC, int NB, typename TO>
 void conv_mma_v(const MmaConvArgs& a, cudaStream_t s) {
   constexpr int R = K / 2, PW = 128 + 2 * R, LDA = KC + 8;
   const size_t smem = (size_t)(K * PW * LDA + K * K * NB * 16 * LDA) * sizeof(bf16);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_conv_mma<K, KC, NB, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    attr = true;
-  }
+  static SmemAttr attr;
+  set_smem(k_conv_mma<K, KC, NB, TO>, smem, attr);
   dim3 grid((unsigned)((long long)a.N * a.H * ((a.W + 127) / 128)), (a.Cout + NB * 16 - 1) / (NB * 16));
   k_conv_mma<K, KC, NB, TO><<<grid, 256, smem, s>>>(a);
   count_launches(1);
@@ -1423,11 +1415,8 @@ template <int MT, int NT>
 void wgrad_mma_v(const WgMmaArgs& a0, cudaStream_t s) {
   WgMmaArgs a = a0;
   constexpr size_t smem = (size_t)(4 * 130 * (8 * NT + 8) + 2 * 128 * (16 * MT + 8)) * sizeof(bf16);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_wgrad_mma<MT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr = true;
-  }
+  static SmemAttr attr;
+  set_smem(k_wgrad_mma<MT, NT>, smem, attr);
   const int xt = (a.W + 127) / 128;
   const unsigned gy = (a.Cin + 8 * NT - 1) / (8 * NT), gz = (a.Cout + 16 * MT - 1) / (16 * MT);
   // one wave of two or three CTAs per SM: each extra strip costs its atomics again
@@ -1490,6 +1479,7 @@ void net_backward(ashrt_unet* u, const float* target, int n, cudaStream_t s) {
   const bool ws = u->cout <= kHeadMaxShared;
   const size_t head_ch = 16 * sizeof(float) + sizeof(double), hs = ws ? u->cout * head_ch : 0;
   auto* head = ws ? k_head_bwd<true> : k_head_bwd<false>;
+  // (beside 26 KB of static shared memory; few heads are this wide: set on every call)
   if (hs > 16 * 1024)
     cudaFuncSetAttribute(head, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(kHeadMaxShared * head_ch));

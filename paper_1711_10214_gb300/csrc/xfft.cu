@@ -460,13 +460,9 @@ template <int LOGN, int C>
 cudaError_t launch_r2c_v(const XfftArgs& a, cudaStream_t s) {
   constexpr int N = 1 << LOGN, T = N * C / 16;
   const size_t smem = (size_t)N * C * sizeof(float2);
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(xfft_r2c_kernel<LOGN, C>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemAttr attr;
+  cudaError_t e = set_smem(xfft_r2c_kernel<LOGN, C>, smem, attr);
+  if (e != cudaSuccess) return e;
   const unsigned grid = tile_grid(a.slabs, a.nt, 2 * C);
   xfft_r2c_kernel<LOGN, C><<<grid, T, smem, s>>>(a);
   return cudaGetLastError();
@@ -494,15 +490,11 @@ cudaError_t launch_r2c_tma(const XfftArgs& a, cudaStream_t s, bool* used) {
   const int nslot = 1 + (mode ? 1 : 0) + (urw ? 1 : 0) + (p2r ? 1 : 0) + (a.ew ? 1 : 0);
   const size_t slot = ((size_t)a.nx * 64 + 127) & ~(size_t)127;
   const size_t smem = 128 + nslot * slot + (size_t)N * C * sizeof(float2) + 16;
-  static int max_smem_set = 0;
-  if ((int)smem > max_smem_set) {
-    cudaError_t e = cudaFuncSetAttribute(xfft_r2c_tma<LOGN>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    max_smem_set = (int)smem;
-  }
+  static SmemAttr attr;
+  cudaError_t e = set_smem(xfft_r2c_tma<LOGN>, smem, attr);
+  if (e != cudaSuccess) return e;
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xfft_r2c_tma<LOGN>, T, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xfft_r2c_tma<LOGN>, T, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaSuccess;
   int dev = 0, sms = 0;
@@ -519,13 +511,9 @@ cudaError_t launch_r2c_tma(const XfftArgs& a, cudaStream_t s, bool* used) {
 template <int LOGN, int C, bool PF, bool NXH>
 cudaError_t launch_c2r_k(const XfftArgs& a, cudaStream_t s, size_t smem) {
   constexpr int N = 1 << LOGN, T = N * C / 16;
-  static size_t attr = 0;
-  if (smem > attr) {
-    cudaError_t e = cudaFuncSetAttribute(xfft_c2r_kernel<LOGN, C, PF, NXH>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr = smem;
-  }
+  static SmemAttr attr;
+  cudaError_t e = set_smem(xfft_c2r_kernel<LOGN, C, PF, NXH>, smem, attr);
+  if (e != cudaSuccess) return e;
   const unsigned grid = tile_grid(a.slabs, a.nt, 2 * C);
   xfft_c2r_kernel<LOGN, C, PF, NXH><<<grid, T, smem, s>>>(a);
   return cudaGetLastError();

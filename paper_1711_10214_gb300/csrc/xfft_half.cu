@@ -223,13 +223,9 @@ template <int LOGN, int C, bool CG>
 cudaError_t r2c_half_k(const XfftArgs& a, cudaStream_t s) {
   constexpr int T = (1 << LOGN) * C / 32;
   const size_t smem = (size_t)(1 << LOGN) * C * sizeof(float2);
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(xfft_r2c_half<LOGN, C, CG>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemAttr attr;
+  cudaError_t e = set_smem(xfft_r2c_half<LOGN, C, CG>, smem, attr);
+  if (e != cudaSuccess) return e;
   xfft_r2c_half<LOGN, C, CG><<<tile_grid(a.slabs, a.nt, 2 * C), T, smem, s>>>(a);
   return cudaGetLastError();
 }
