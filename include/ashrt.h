@@ -342,17 +342,22 @@ ashrt_status ashrt_sort_gathers(const float* src_dev, int n0, int n1, int nt, fl
  * to Nt = 512, 6 at Nt = 1024 and 4096 and for small batches at Nt = 2048, 9 for
  * large ones there, and between them the forward of 9 with the adjoint of 6)
  * and the trace-axis FFT column tile (16 or 8 columns for Nx <= 512) -- and
- * keeps the fastest in the plan; the plan's current choice is timed first and
- * another one replaces it only when it is more than 2% faster, so variants
- * within timing noise of each other do not flip from run to run.  With cache_path (a JSON-lines file, one object per
- * device and problem shape) a cached choice is reused without timing and new
- * choices are appended.  Allocates and frees temporary buffers; synchronises.
- * The chosen variants are returned in rows_minb / xfft_cols (may be NULL).
- * Every variant computes the same operator.
+ * keeps the fastest in the plan; the choice by rule is timed first and another
+ * one replaces it only when it is more than 2% faster, so variants within timing
+ * noise of each other do not flip from run to run.  A variant other than the
+ * rule's holds for calls of `batch` gathers, calls of another number go by the
+ * rule; the column tile holds for all.  With cache_path (a JSON-lines file, one
+ * object per device and problem shape) a cached choice is reused without timing
+ * and new choices are appended.  Allocates and frees temporary buffers;
+ * synchronises.  The chosen variants are returned in rows_minb / xfft_cols (may
+ * be NULL); where the rule was kept and mixes two forms, its forward's.
+ * Every variant computes the same operator.  Form, panel split and trace-axis
+ * kernel follow the size of a launch, so the last bits of a gather's result may
+ * depend on the number of gathers in the call; a set variant fixes the form alone.
  */
 ashrt_status ashrt_plan_autotune(ashrt_plan* plan, int batch, const char* cache_path,
                                  int* rows_minb, int* xfft_cols);
-/* Sets the variants directly (rows_minb 1..9, xfft_cols 8 or 16); register
+/* Sets the variants directly, for every batch (rows_minb 1..9, xfft_cols 8 or 16); register
  * caps and column tiles that do not apply to the plan's sizes fall back to the
  * default kernel; rows_minb 4..9 on an Nt other than 1024, 2048 or 4096 is
  * ASHRT_EINVAL. */

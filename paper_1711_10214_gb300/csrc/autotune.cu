@@ -2,7 +2,9 @@
 // cap, i.e. resident CTAs per SM, or their radix-16 form, and the trace-axis
 // FFT column tile) by timing
 // forward+adjoint operator pairs on the plan's own sizes, and keeps the choice
-// in a JSON-lines cache keyed by device and problem shape.
+// in a JSON-lines cache keyed by device and problem shape.  The choice by rule
+// (rows_variant) is one of those timed; another variant holds for the batch that
+// it was timed with.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -27,17 +29,19 @@ __global__ void k_fill_hash(float* x, long long n, unsigned seed) {
   }
 }
 
+// (rows=2: the second generation of row kernels; times of earlier ones do not hold)
 std::string tune_key(const ashrt_plan* p, int batch) {
   cudaDeviceProp prop;
   char name[256] = "unknown";
   if (cudaGetDeviceProperties(&prop, p->device) == cudaSuccess) snprintf(name, sizeof(name), "%s", prop.name);
   char buf[512];
-  snprintf(buf, sizeof(buf), "%s|variants=9|nt=%d|nx=%d|Nt=%d|Nx=%d|P=%d|shift=%d|B=%d", name,
+  snprintf(buf, sizeof(buf), "%s|rows=2|nt=%d|nx=%d|Nt=%d|Nx=%d|P=%d|shift=%d|B=%d", name,
            p->nt, p->nx,
            p->Nt, p->Nx, p->P, p->shift ? 1 : 0, batch);
   return buf;
 }
 
+// minb: 0 where the line says that the rule was the fastest.
 bool cache_lookup(const char* path, const std::string& key, int* minb, int* cols) {
   if (!path) return false;
   FILE* f = fopen(path, "r");
@@ -50,18 +54,28 @@ bool cache_lookup(const char* path, const std::string& key, int* minb, int* cols
     const char* a = strstr(line, "\"rows_minb\": ");
     const char* b = strstr(line, "\"xfft_cols\": ");
     if (a && b && sscanf(a + 13, "%d", minb) == 1 && sscanf(b + 13, "%d", cols) == 1) found = true;
+    if (found && strstr(line, "\"rule\": 1")) *minb = 0;
   }
   fclose(f);
   return found;
 }
 
-void cache_store(const char* path, const std::string& key, int minb, int cols, double ms) {
+// minb: the variant as reported, also where it was left to the rule.
+void cache_store(const char* path, const std::string& key, int minb, bool rule, int cols, double ms) {
   if (!path) return;
   FILE* f = fopen(path, "a");
   if (!f) return;
-  fprintf(f, "{\"key\": \"%s\", \"rows_minb\": %d, \"xfft_cols\": %d, \"pair_ms\": %.4f}\n",
-          key.c_str(), minb, cols, ms);
+  fprintf(f, "{\"key\": \"%s\", \"rows_minb\": %d, \"rule\": %d, \"xfft_cols\": %d, \"pair_ms\": %.4f}\n",
+          key.c_str(), minb, rule ? 1 : 0, cols, ms);
   fclose(f);
+}
+
+// Keeps variant minb (0: the rule's, for every batch) for `batch` gathers; returns the
+// variant to report, 1..9 (the rule's mixed form 10 has the forward of 9).
+int keep_variant(ashrt_plan* p, int minb, int batch) {
+  p->rows_minb = minb;
+  p->tuned_batch = minb ? batch : 0;
+  return std::min(9, ashrt::rows_variant(p, batch));
 }
 
 }  // namespace
@@ -77,7 +91,7 @@ extern "C" ashrt_status ashrt_plan_autotune(ashrt_plan* p, int batch, const char
   const std::string key = tune_key(p, batch);
   int minb = 0, cols = p->xfft_cols;
   if (cache_lookup(cache_path, key, &minb, &cols)) {
-    p->rows_minb = minb;
+    minb = keep_variant(p, minb, batch);
     p->xfft_cols = cols;
     if (rows_minb) *rows_minb = minb;
     if (xfft_cols) *xfft_cols = cols;
@@ -124,11 +138,11 @@ extern "C" ashrt_status ashrt_plan_autotune(ashrt_plan* p, int batch, const char
     return err;
   };
 
-  // the plan's default variant is timed first and kept unless another one is
-  // faster by more than 2% (timing noise does not flip the choice)
-  // (the rule's mixed form 10 is not a choice of its own: 9 stands for it)
-  const int def_minb = std::min(9, rows_variant(p, batch));
-  std::vector<int> minbs = {def_minb};
+  // the choice by rule (0) is timed first and kept unless another one is faster by
+  // more than 2% (timing noise does not flip the choice)
+  p->rows_minb = 0;
+  const int by_rule = rows_variant(p, batch);
+  std::vector<int> minbs = {0};
   std::vector<int> cand = {3};
   if (p->logNt >= 9 && p->logNt <= 11) cand = {3, 2, 1};
   if (rows16_supported(p->logNt) && p->tw_t16) {
@@ -136,24 +150,24 @@ extern "C" ashrt_status ashrt_plan_autotune(ashrt_plan* p, int batch, const char
     if (p->logNt == 11) cand.push_back(9);
   }
   for (int v : cand)
-    if (v != def_minb) minbs.push_back(v);
+    if (v != by_rule) minbs.push_back(v);
   std::vector<int> colss = {16};
   if (p->logNx <= 9) colss = {16, 8};
   double best = 1e30;
   int best_minb = minbs[0], best_cols = colss[0];
   for (int mb : minbs) {
-    p->rows_minb = mb;
+    keep_variant(p, mb, batch);
     p->xfft_cols = best_cols;
     double ms = 0.0;
     e = time_pair(&ms);
     if (e != cudaSuccess) break;
-    if (ms < (mb == def_minb ? best : 0.98 * best)) {
+    if (ms < (mb == 0 ? best : 0.98 * best)) {
       best = ms;
       best_minb = mb;
     }
   }
   for (size_t i = 1; i < colss.size() && e == cudaSuccess; ++i) {
-    p->rows_minb = best_minb;
+    keep_variant(p, best_minb, batch);
     p->xfft_cols = colss[i];
     double ms = 0.0;
     e = time_pair(&ms);
@@ -163,14 +177,14 @@ extern "C" ashrt_status ashrt_plan_autotune(ashrt_plan* p, int batch, const char
     }
   }
   cleanup();
-  p->rows_minb = best_minb;
+  const int reported = keep_variant(p, best_minb, batch);
   p->xfft_cols = best_cols;
   if (e != cudaSuccess) {
     set_error("ashrt_plan_autotune: timing failed: %s", cudaGetErrorString(e));
     return ASHRT_ECUDA;
   }
-  cache_store(cache_path, key, best_minb, best_cols, best);
-  if (rows_minb) *rows_minb = best_minb;
+  cache_store(cache_path, key, reported, best_minb == 0, best_cols, best);
+  if (rows_minb) *rows_minb = reported;
   if (xfft_cols) *xfft_cols = best_cols;
   return ASHRT_OK;
 }
@@ -186,6 +200,7 @@ extern "C" ashrt_status ashrt_plan_set_variant(ashrt_plan* p, int rows_minb, int
     return ASHRT_EINVAL;
   }
   p->rows_minb = rows_minb;
+  p->tuned_batch = 0;
   p->xfft_cols = xfft_cols;
   return ASHRT_OK;
 }

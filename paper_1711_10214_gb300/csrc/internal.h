@@ -201,8 +201,9 @@ struct ashrt_plan {
   int with_solver = 0;
   ashrt_opts opts{};
   bool shift = false;        // any nonzero tau0
-  int rows_minb = 3;         // row-kernel variant 1..9 (set or autotuned; see
+  int rows_minb = 0;         // row-kernel variant 1..9 (set or autotuned; see
                              // ashrt_plan_autotune), 0: by rule (rows_variant)
+  int tuned_batch = 0;       // the only batch that rows_minb holds for, 0: for every batch
   int xfft_cols = 16;
   // device tables
   float2* tw_t = nullptr;

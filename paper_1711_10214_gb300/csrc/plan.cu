@@ -188,7 +188,8 @@ size_t data_elems(const ashrt_plan* p) { return (size_t)p->nr * p->nt; }
 //     table read between two gathers, which wins once pairs alone fill the chip:
 //     12 gathers (R = 3084) 511 against 518, 64 gathers 2593 against 2491.
 int rows_variant(const ashrt_plan* p, int batch) {
-  if (p->rows_minb) return p->rows_minb;
+  if (p->rows_minb && (!p->tuned_batch || p->tuned_batch == batch)) return p->rows_minb;
+  if (!p->tw_t16) return 3;
   if (p->logNt != 11 || batch < 2) return 6;
   return (long long)batch * p->Lh <= 3600 ? 10 : 9;
 }
@@ -555,7 +556,6 @@ static ashrt_status plan_create_impl(ashrt_plan** out, int nt, int nx, double dt
     std::vector<float2> tw16(twiddle_table_len(p->logNt, 4));
     build_twiddle_table(p->logNt, tw16.data(), 4);
     chk(upload(&p->tw_t16, tw16, &total));
-    p->rows_minb = 0;   // by rule (rows_variant) until a variant is set or tuned
   }
   chk(upload(&p->wt, wt, &total));
   chk(upload(&p->kmin, kmin, &total));
