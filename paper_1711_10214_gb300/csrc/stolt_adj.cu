@@ -124,9 +124,10 @@ cudaError_t launch_adj_vh(const RowArgs& a, cudaStream_t s) {
   const size_t smem = (size_t)2 * N * sizeof(float4) + (size_t)a.atab_ld * sizeof(uint2);
   cudaError_t e = set_smem(stolt_adj_rows<LOGN, SHIFT, MINB, HALF>, smem_cap<LOGN>(false), attr);
   if (e != cudaSuccess) return e;
-  // rows of Nt <= 512 may fill an SM with more than MINB CTAs
-  const int n = rows_split((long long)a.Lh * ((a.batch + 1) / 2), a.P, LOGN <= 9 ? 8 : MINB,
-                           false);
+  // rows of Nt <= 512 (one or two warps) fill an SM with as many CTAs as their registers allow
+  const int n = rows_split((long long)a.Lh * ((a.batch + 1) / 2), a.P,
+                           LOGN <= 8 ? 15 : LOGN == 9 ? 9 : MINB,
+                           LOGN <= 8 ? 14.0 : LOGN == 9 ? 10.0 : 3.0, false);
   stolt_adj_rows<LOGN, SHIFT, MINB, HALF>
       <<<dim3(a.Lh, (a.batch + 1) / 2, n), N / 8, smem, s>>>(a);
   return cudaGetLastError();

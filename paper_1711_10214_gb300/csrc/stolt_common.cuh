@@ -211,33 +211,40 @@ __device__ __forceinline__ void panel_chunk(int P, int n, int z, int& p0, int& p
 
 // Chunks a row's panels are split into, so that few rows (small batches,
 // narrow gathers) still fill the chip: 1, 2, 4 or 8.  `ctas` rows of P panels
-// each run as ctas x n CTAs, `res` of them resident per SM.  A panel takes a
-// CTA about a + b k with k CTAs on its SM (a: the latency of its dependent
-// passes, b: its share of the shared-memory pipe; a/b about 2.5 in all the row
-// kernels: e.g. the single-gather forward at Nt 2048 1.2 us and 0.5 us), and
-// every chunk costs about one and a half panels more (setup and the extra
-// data-row transform of the adjoint, or the sum over the chunks of the
-// forward), so the candidate with the smallest
-//   waves(n) (P / n + 1.5) (2.5 + k(n))
-// is taken.  `ordered` (the forward): up to eight panels are split one to a
-// CTA or not at all, so that the partial sums, added in rank order, are those
-// of the unsplit loop to the last bit.  Forward / adjoint rows per launch, before and after: 1 gather
-// 256 x 64, 8 panels (65 rows) 16.3 / 18.2 -> 11.0 / 10.4 us; 2 gathers
-// 181 x 455, 25 panels (513 rows of pairs) 51 / 54 -> 45 / 41 us; 1 gather
+// each run as ctas x n CTAs, `res` of them resident per SM.  With k CTAs on its SM a
+// panel takes about (a^4 + k^4)^(1/4) times a constant: the latency of its dependent
+// passes until `a` CTAs fill the pipe that bounds the kernel (shared memory or issue),
+// its share of that pipe beyond.  A CTA costs about one and a half panels more (setup,
+// and the extra data-row transform of the adjoint), and the forward's sum over the
+// chunks (`sum`) as much again, so the candidate with the smallest
+//   waves(n) (P / n + 1.5 [+ 1.5]) (a^4 + k(n)^4)^(1/4)
+// is taken, if it is 5% below the unsplit one; waves(n) is the whole number, or with
+// `ragged` the mean of it and the fraction (CTAs short enough to even out the last wave:
+// adjoint, 1 gather 1024 x 417, 72 panels 435 -> 380 us).  With the residencies and the values
+// of `a` at the launches, fitted to 1600 rows launches of 65 to 3084 rows, 1 to 32 panels
+// and Nt 64 to 4096, the choice is within 1% of the best on average and at most 1.12 times
+// the unsplit launch (a line in k without the sum's cost, as it was: 1.6 times, 26.7 and
+// 41.9 us for 12 gathers 100 x 256, 9 panels).  `sum` (the forward) also splits up
+// to eight panels one to a CTA or not at all, so that the partial sums, added in rank
+// order, are those of the unsplit loop to the last bit.  Forward / adjoint rows per launch,
+// whole and split: 1 gather 256 x 64, 8 panels (65 rows) 16.3 / 18.2 -> 11.0 / 10.4 us;
+// 2 gathers 181 x 455, 25 panels (513 rows of pairs) 51 / 54 -> 45 / 41 us; 1 gather
 // 1024 x 256, 32 panels (257 rows, single-gather form) 75 / 82 -> 62 / 60 us;
 // 2 gathers 1024 x 128, 192 panels (258 rows) 451 / 555 -> 349 / 347 us, as 129
 // pairs 459 -> 224 us forward.
-inline int rows_split(long long ctas, int P, int res, bool ordered) {
+inline int rows_split(long long ctas, int P, int res, double a, bool sum, bool ragged = false) {
   constexpr int kSms = 152;
   int best = 1;
   double best_t = 0.0;
-  const bool whole = ordered && P <= 8;
+  const bool whole = sum && P <= 8;
   for (int n = 1; n <= 8 && n <= P; n = whole && n < P ? P : 2 * n) {
     const double per_sm = (double)((ctas * n + kSms - 1) / kSms);
     const double k = per_sm < res ? per_sm : res;
-    const double waves = std::ceil(per_sm / k);
-    const double t = waves * ((P + n - 1) / n + 1.5) * (2.5 + k);
-    if (n == 1 || t < 0.95 * best_t) {
+    const double part = (double)(ctas * n) / kSms / k, whole_waves = std::ceil(per_sm / k);
+    const double waves = ragged ? 0.5 * (whole_waves + (part > 1.0 ? part : 1.0)) : whole_waves;
+    const double ends = sum && n > 1 ? 3.0 : 1.5;
+    const double t = waves * ((P + n - 1) / n + ends) * std::pow(a * a * a * a + k * k * k * k, 0.25);
+    if (n == 1 || t < (ragged ? 0.96 : 0.95) * best_t) {
       best = n;
       best_t = t;
     }

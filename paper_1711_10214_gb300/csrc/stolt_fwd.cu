@@ -146,7 +146,8 @@ cudaError_t launch_fwd_vh(const RowArgs& a0, cudaStream_t s) {
   const dim3 grid(a.Lh, (a.batch + 1) / 2);
   if constexpr (LOGN <= 9) {
     // longer rows have single-gather kernels for batches this small
-    a.psplit = rows_split((long long)grid.x * grid.y, a.P, 8, true);
+    a.psplit = rows_split((long long)grid.x * grid.y, a.P, LOGN <= 8 ? 12 : 8,
+                          LOGN <= 8 ? 6.0 : 5.0, true);
     if (a.psplit > 1) {
       static SmemAttr attr;
       cudaError_t e = set_smem(stolt_fwd_rows<LOGN, SHIFT, MINB, HALF, true>, smem_cap<LOGN>(true),

@@ -831,11 +831,9 @@ cudaError_t launch_fwd32_tm(const RowArgs& a0, cudaStream_t s) {
   constexpr int N = 1 << 11;
   RowArgs a = a0;
   const dim3 grid(a.Lh, (a.batch + 1) / 2);
-  // two waves of CTAs and more are not split: the set-up of each (the twiddles) costs
-  // more than the fuller last wave gives (16 gathers, 2056 CTAs, 32 panels: 541 split
-  // against 504; 6 gathers 1024 x 128, 387 CTAs, 192 panels: 586 against 698)
-  const long long ctas = (long long)grid.x * grid.y;
-  a.psplit = ctas < 2 * 152 * 4 ? rows_split(ctas, a.P, 4, true) : 1;
+  // (16 gathers, 2056 CTAs, 32 panels: 541 us split against 504, the rule leaves them whole;
+  // 6 gathers 1024 x 128, 387 CTAs, 192 panels: 586 against 698)
+  a.psplit = rows_split((long long)grid.x * grid.y, a.P, 4, 3.0, true);
   static_assert(4 * kSide32 * sizeof(float2) >= N * sizeof(float4), "the final transform's row");
   const size_t smem = 4 * kSide32 * sizeof(float2) + (size_t)a.taps_ld * sizeof(unsigned) + 16;
   if (a.psplit > 1)

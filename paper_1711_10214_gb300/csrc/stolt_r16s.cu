@@ -237,7 +237,8 @@ template <int LOGN, bool SHIFT, bool HALF>
 cudaError_t launch_fwd16s_h(const RowArgs& a0, cudaStream_t s) {
   constexpr int N = 1 << LOGN;
   RowArgs a = a0;
-  a.psplit = rows_split((long long)a.batch * a.Lh, a.P, r16s_minb_fwd<LOGN>(), true);
+  a.psplit = rows_split((long long)a.batch * a.Lh, a.P, r16s_minb_fwd<LOGN>(),
+                        LOGN == 10 ? 5.0 : LOGN == 11 ? 3.0 : 2.0, true);
   const size_t smem = (size_t)(N + a.ld) * sizeof(float2), cap = (size_t)2 * N * sizeof(float2);
   if (a.psplit > 1) {
     static SmemAttr attr;
@@ -266,7 +267,8 @@ cudaError_t launch_adj16s_h(const RowArgs& a, cudaStream_t s) {
   const size_t smem = (size_t)2 * N * sizeof(float2);
   cudaError_t e = set_smem(stolt_adj_rows16s<LOGN, SHIFT, HALF>, smem, attr);
   if (e != cudaSuccess) return e;
-  const int n = rows_split((long long)a.batch * a.Lh, a.P, r16s_minb_adj<LOGN>(), false);
+  const int n = rows_split((long long)a.batch * a.Lh, a.P, r16s_minb_adj<LOGN>(),
+                           LOGN == 10 ? 5.0 : LOGN == 11 ? 3.0 : 1.75, false, LOGN == 11);
   stolt_adj_rows16s<LOGN, SHIFT, HALF><<<dim3(a.batch, a.Lh, n), N / 16, smem, s>>>(a);
   return cudaGetLastError();
 }
