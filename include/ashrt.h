@@ -338,9 +338,9 @@ ashrt_status ashrt_sort_gathers(const float* src_dev, int n0, int n1, int nt, fl
  * pair forward with that adjoint, 9: as 5 with the forward's per-bin sums in
  * tensor memory instead of registers (Nt = 2048 only, four CTAs per SM
  * instead of three; on other lengths the same kernels as 5); without a set or
- * tuned variant each call takes the form measured fastest for its batch: 3 up
- * to Nt = 512, 6 at Nt = 1024 and 4096 and for small batches at Nt = 2048, 9 for
- * large ones there, and between them the forward of 9 with the adjoint of 6)
+ * tuned variant each call takes the form measured fastest for its sizes: 3 up
+ * to Nt = 512, 6 at Nt = 1024 and 4096 and for few rows and panels at Nt = 2048, 9
+ * for many there, and between them the forward of 9 with the adjoint of 6)
  * and the trace-axis FFT column tile (16 or 8 columns for Nx <= 512) -- and
  * keeps the fastest in the plan; the choice by rule is timed first and another
  * one replaces it only when it is more than 2% faster, so variants within timing

@@ -181,17 +181,29 @@ size_t data_elems(const ashrt_plan* p) { return (size_t)p->nr * p->nt; }
 //     against 4790 / 5258.
 //   Nt 1024: the single-gather form: 16 panels, 129 rows, 16 gathers 95 / 94
 //     against 121 / 111 (4), 64 gathers 347 / 338 against 336 / 369.
-//   Nt 2048: the pair form's forward (9) from two gathers on: 32 panels, 129 rows:
-//     1 gather 37 single against 53, 2 gathers 65 against 52; 257 rows: 2 gathers 110
-//     against 88, 3 164 against 151, 4 192 against 152; 192 panels, 129 rows, 2
-//     gathers 350 against 224.  The adjoint's pair form shares each twiddle and
-//     table read between two gathers, which wins once pairs alone fill the chip:
-//     12 gathers (R = 3084) 511 against 518, 64 gathers 2593 against 2491.
+//   Nt 2048, forward: the pair form (9) shares each table read between two gathers but
+//     sets up its twiddles per CTA and splits fewer rows, so it needs work enough, R P from
+//     2400 on (more where an odd batch leaves half a pair empty).  Single and pair: R 258,
+//     4 panels 14.7 and 20, 32 panels 105 and 85; R 1032, 2 panels 24 and 24.5; R 66, 32
+//     panels 31 and 31; R 4128, 32 panels 870 and 620.  One panel: single up to R 4096
+//     (8.6 and 12.3 at R 258), the radix-16 pair (8) beyond (151 against 156 at 16416).
+//   Nt 2048, adjoint: the single-gather form until pairs alone fill the chip several times
+//     over, and with few panels always: 12 gathers (R 3084), 32 panels 511 against 518,
+//     64 gathers 2593 against 2491; 8 panels 1.00 to 1.05 times as fast up to R 16416.
+//     With asymptote shifts a pair shares the phase table too: from 250 pairs of rows on,
+//     but for a second wave that is nearly empty (three CTAs per SM) and three gathers (a
+//     quarter of the rows empty): 24 panels, R 774 / 3084 / 16416 1.17 / 1.20 / 1.25
+//     times as fast in pairs, R 1040 0.92 times.
 int rows_variant(const ashrt_plan* p, int batch) {
   if (p->rows_minb && (!p->tuned_batch || p->tuned_batch == batch)) return p->rows_minb;
   if (!p->tw_t16) return 3;
   if (p->logNt != 11 || batch < 2) return 6;
-  return (long long)batch * p->Lh <= 3600 ? 10 : 9;
+  const long long R = (long long)batch * p->Lh, pairs = (batch + 1) / 2 * (long long)p->Lh;
+  if (p->P == 1) return R > 4096 ? 8 : 6;
+  if (R * p->P * R < 2400 * 2 * pairs) return 6;   // R P, times the share of the pairs in use
+  const bool adj_pair = p->shift ? batch != 3 && pairs >= 250 && (pairs <= 3 * 152 || pairs >= 640)
+                                 : p->P > 8 && R > 3600;
+  return adj_pair ? 9 : 10;
 }
 
 // ---------------------------------------------------------------------------
