@@ -516,16 +516,6 @@ int tc_tile(int K, int cout) {
   }
 }
 
-// ---------------------------------------------------------------------------
-// Tensor-core forward convolution (mma.sync m16n8k16, BF16 operands, FP32
-// accumulation) for layers whose input channels are a multiple of 16: an
-// implicit GEMM with M = pixels, N = output channels, K = taps x input
-// channels.  CTA: 128 consecutive pixels of one image row x NB*16 output
-// channels, 8 warps of 16 pixels each.  Per chunk of KC input channels the
-// three input rows (130 pixels with the halo) and the weights of all taps are
-// staged in shared memory (rows padded by 8 elements against bank conflicts)
-// and consumed by ldmatrix fragments; bias, ReLU and the BF16 (or FP32)
-// store are fused into the epilogue.
 __device__ __forceinline__ void ldsm_x4(uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3,
                                         const void* p) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];\n"
@@ -542,90 +532,58 @@ __device__ __forceinline__ void mma_bf16(float* c, uint32_t a0, uint32_t a1, uin
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-struct MmaConvArgs {
-  Tensor in;             // bf16 NHWC slice, ps and off multiples of 8
-  const bf16* w;         // [K*K][Cout][Cin]
-  const float* bias;     // [Cout]
-  Tensor out;            // bf16 or fp32 NHWC slice
-  int N, H, W, Cin, Cout, relu;
-};
-
-template <int K, int KC, int NB, typename TO>
-__global__ void __launch_bounds__(256, 2) k_conv_mma(MmaConvArgs a) {
-  constexpr int R = K / 2, PW = 128 + 2 * R, LDA = KC + 8, NT = NB * 16, TAPS = K * K;
-  extern __shared__ __align__(16) unsigned char smc[];
-  bf16* xs = (bf16*)smc;                              // [K rows][PW px][LDA]
-  bf16* ws = xs + K * PW * LDA;                       // [TAPS][NT co][LDA]
+// The head where it is wider than the tcgen05 tiles (mma.sync m16n8k16, BF16 operands,
+// FP32 accumulation): out [pixels][Cout] = bias + in [pixels][16] w^T, w [Cout][16].  CTA:
+// 128 pixels x 16 NB output channels, 8 warps of 16 pixels each, both operands staged in
+// shared memory (rows padded by 8 elements against bank conflicts).
+template <int NB>
+__global__ void __launch_bounds__(256, 2) k_head_mma(const bf16* __restrict__ in,
+                                                     const bf16* __restrict__ w,
+                                                     const float* __restrict__ bias, float* out,
+                                                     long long npix, int Cout) {
+  constexpr int LD = 24, NT = NB * 16;
+  __shared__ __align__(16) bf16 xs[128 * LD], ws[NT * LD];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int xt = (a.W + 127) / 128;
-  const int row = blockIdx.x / xt;
-  const int x0 = (blockIdx.x % xt) * 128;
-  const int n = row / a.H, y = row % a.H;
+  const long long p0 = blockIdx.x * 128LL;
   const int co0 = blockIdx.y * NT;
-  const bf16* in = (const bf16*)a.in.p;
+  {
+    const int v = tid & 1, px = tid >> 1;          // 16-byte vectors of 8 channels
+    uint4 val = make_uint4(0u, 0u, 0u, 0u);
+    if (p0 + px < npix) val = *(const uint4*)(in + (p0 + px) * 16 + 8 * v);
+    *(uint4*)(xs + px * LD + 8 * v) = val;
+  }
+  for (int e = tid; e < NT * 2; e += 256) {
+    const int v = e & 1, c = e >> 1;
+    uint4 val = make_uint4(0u, 0u, 0u, 0u);
+    if (co0 + c < Cout) val = *(const uint4*)(w + (co0 + c) * 16 + 8 * v);
+    *(uint4*)(ws + c * LD + 8 * v) = val;
+  }
+  __syncthreads();
   float acc[2 * NB][4];
 #pragma unroll
   for (int j = 0; j < 2 * NB; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-
-  for (int ci0 = 0; ci0 < a.Cin; ci0 += KC) {
-    // stage the input rows: 16-byte vectors of 8 channels
-    constexpr int VPX = KC / 8;
-    for (int e = tid; e < K * PW * VPX; e += 256) {
-      const int v = e % VPX, px = (e / VPX) % PW, r = e / (VPX * PW);
-      const int yy = y + r - R, xx = x0 + px - R;
-      uint4 val = make_uint4(0u, 0u, 0u, 0u);
-      if (yy >= 0 && yy < a.H && xx >= 0 && xx < a.W)
-        val = *(const uint4*)(in + (((long long)n * a.H + yy) * a.W + xx) * a.in.ps + a.in.off +
-                              ci0 + 8 * v);
-      *(uint4*)(xs + (r * PW + px) * LDA + 8 * v) = val;
-    }
-    for (int e = tid; e < TAPS * NT * VPX; e += 256) {
-      const int v = e % VPX, c = (e / VPX) % NT, tap = e / (VPX * NT);
-      uint4 val = make_uint4(0u, 0u, 0u, 0u);
-      if (co0 + c < a.Cout)
-        val = *(const uint4*)(a.w + ((long long)tap * a.Cout + co0 + c) * a.Cin + ci0 + 8 * v);
-      *(uint4*)(ws + (tap * NT + c) * LDA + 8 * v) = val;
-    }
-    __syncthreads();
+  uint32_t a0, a1, a2, a3;
+  ldsm_x4(a0, a1, a2, a3, xs + (warp * 16 + (lane & 15)) * LD + ((lane >> 4) << 3));
 #pragma unroll
-    for (int tap = 0; tap < TAPS; ++tap) {
-      const int dy = tap / K, dx = tap % K;
-#pragma unroll
-      for (int kk = 0; kk < KC; kk += 16) {
-        uint32_t a0, a1, a2, a3;
-        // A: rows = the warp's 16 pixels (shifted by dx), k = channels kk..kk+15
-        const int ar = lane & 15, ak = kk + ((lane >> 4) << 3);
-        ldsm_x4(a0, a1, a2, a3, xs + (dy * PW + warp * 16 + ar + dx) * LDA + ak);
-#pragma unroll
-        for (int nb = 0; nb < NB; ++nb) {
-          // B: two n8 blocks of 16 output channels, k = channels kk..kk+15
-          uint32_t b0, b1, b2, b3;
-          const int bn = nb * 16 + (lane & 7) + ((lane >> 4) << 3), bk = kk + (((lane >> 3) & 1) << 3);
-          ldsm_x4(b0, b1, b2, b3, ws + (tap * NT + bn) * LDA + bk);
-          mma_bf16(acc[2 * nb], a0, a1, a2, a3, b0, b1);
-          mma_bf16(acc[2 * nb + 1], a0, a1, a2, a3, b2, b3);
-        }
-      }
-    }
-    __syncthreads();
+  for (int nb = 0; nb < NB; ++nb) {
+    uint32_t b0, b1, b2, b3;                       // two n8 blocks of 16 output channels
+    const int bn = nb * 16 + (lane & 7) + ((lane >> 4) << 3), bk = ((lane >> 3) & 1) << 3;
+    ldsm_x4(b0, b1, b2, b3, ws + bn * LD + bk);
+    mma_bf16(acc[2 * nb], a0, a1, a2, a3, b0, b1);
+    mma_bf16(acc[2 * nb + 1], a0, a1, a2, a3, b2, b3);
   }
-  // epilogue: c0, c1 at (pixel g, channels 2t, 2t+1), c2, c3 at pixel g + 8
+  // c0, c1 at (pixel g, channels 2t, 2t+1), c2, c3 at pixel g + 8
   const int g = lane >> 2, t = lane & 3;
-  TO* out = (TO*)a.out.p;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    const int xx = x0 + warp * 16 + g + 8 * h;
-    if (xx >= a.W) continue;
-    const long long pix = ((long long)n * a.H + y) * a.W + xx;
+    const long long p = p0 + warp * 16 + g + 8 * h;
+    if (p >= npix) continue;
 #pragma unroll
     for (int j = 0; j < 2 * NB; ++j) {
-      const int co = co0 + 8 * j + 2 * t;
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        if (co + u >= a.Cout) continue;
-        float v = acc[j][2 * h + u] + a.bias[co + u];
-        if (a.relu) v = fmaxf(v, 0.f);
-        st_f(out, pix * a.out.ps + a.out.off + co + u, v);
+        const int co = co0 + 8 * j + 2 * t + u;
+        if (co < Cout) out[p * Cout + co] = acc[j][2 * h + u] + bias[co];
       }
     }
   }
@@ -1129,52 +1087,20 @@ bool conv_tc(Tensor in, const bf16* w, const float* bias, Tensor out, int N, int
   }
 }
 
-template <int K, int KC, int NB, typename TO>
-void conv_mma_v(const MmaConvArgs& a, cudaStream_t s) {
-  constexpr int R = K / 2, PW = 128 + 2 * R, LDA = KC + 8;
-  const size_t smem = (size_t)(K * PW * LDA + K * K * NB * 16 * LDA) * sizeof(bf16);
-  static SmemAttr attr;
-  set_smem(k_conv_mma<K, KC, NB, TO>, smem, attr);
-  dim3 grid((unsigned)((long long)a.N * a.H * ((a.W + 127) / 128)), (a.Cout + NB * 16 - 1) / (NB * 16));
-  k_conv_mma<K, KC, NB, TO><<<grid, 256, smem, s>>>(a);
+// The wide head (more than 48 channels): the widest tile that divides its channels.
+template <int NB>
+void head_mma_v(const bf16* in, const bf16* w, const float* bias, float* out, long long npix,
+                int Cout, cudaStream_t s) {
+  const dim3 grid((unsigned)((npix + 127) / 128), (Cout + NB * 16 - 1) / (NB * 16));
+  k_head_mma<NB><<<grid, 256, 0, s>>>(in, w, bias, out, npix, Cout);
   count_launches(1);
 }
-
-// Tensor-core forward convolution (input channels a multiple of 16, channel
-// strides and offsets multiples of 8): picks the channel chunk and the
-// output-channel tile from the layer's sizes.
-template <int K, typename TO>
-void conv_mma(Tensor in, const bf16* w, const float* bias, Tensor out, int N, int H, int W,
-              int Cin, int Cout, int relu, cudaStream_t s) {
-  MmaConvArgs a;
-  a.in = in;
-  a.w = w;
-  a.bias = bias;
-  a.out = out;
-  a.N = N;
-  a.H = H;
-  a.W = W;
-  a.Cin = Cin;
-  a.Cout = Cout;
-  a.relu = relu;
-  const bool kc32 = Cin % 32 == 0;
-  const int nb = Cout % 64 == 0 ? 4 : Cout % 48 == 0 ? 3 : Cout % 32 == 0 ? 2 : Cout <= 16 ? 1
-               : std::min(4, (Cout + 15) / 16);
-  if (kc32) {
-    switch (nb) {
-      case 1: conv_mma_v<K, 32, 1, TO>(a, s); break;
-      case 2: conv_mma_v<K, 32, 2, TO>(a, s); break;
-      case 3: conv_mma_v<K, 32, 3, TO>(a, s); break;
-      default: conv_mma_v<K, 32, 4, TO>(a, s); break;
-    }
-  } else {
-    switch (nb) {
-      case 1: conv_mma_v<K, 16, 1, TO>(a, s); break;
-      case 2: conv_mma_v<K, 16, 2, TO>(a, s); break;
-      case 3: conv_mma_v<K, 16, 3, TO>(a, s); break;
-      default: conv_mma_v<K, 16, 4, TO>(a, s); break;
-    }
-  }
+void head_mma(const bf16* in, const bf16* w, const float* bias, float* out, long long npix, int Cout,
+              cudaStream_t s) {
+  if (Cout % 64 == 0) head_mma_v<4>(in, w, bias, out, npix, Cout, s);
+  else if (Cout % 48 == 0) head_mma_v<3>(in, w, bias, out, npix, Cout, s);
+  else if (Cout % 32 == 0) head_mma_v<2>(in, w, bias, out, npix, Cout, s);
+  else head_mma_v<4>(in, w, bias, out, npix, Cout, s);
 }
 
 // rms[g] of the n input gathers x [n][per]
@@ -1230,8 +1156,7 @@ void net_forward(ashrt_unet* u, int n, cudaStream_t s, const HeadOut& head) {
                          none, head)) {
     // a head wider than the tcgen05 tiles: pixel-major, then to its planar place
     const long long P = (long long)H * W;
-    conv_mma<1, float>(T_(u->d1b, c0), L[14].c.wn, B(14), T_(u->ynhwc, u->cout), n, H, W, c0, u->cout,
-                       0, s);
+    head_mma(u->d1b, L[14].c.wn, B(14), u->ynhwc, P * n, u->cout, s);
     k_unpack_out<<<grid1d(P * n), 256, 0, s>>>(u->ynhwc, head, P, u->cout, n);
     count_launches(1);
   }
