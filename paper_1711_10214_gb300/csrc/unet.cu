@@ -678,8 +678,10 @@ Tensor T_(void* p, int ps, int off = 0) {
 //     lanes 32 (w mod 4)..+31, alternate column groups), fuse bias, ReLU or the
 //     mask and store, while the next tile accumulates in the other half of TMEM.
 // Every wait is bounded; one that runs out ends its role, then the others', and
-// sets the error flag.  What bounds a layer is the tensor pipe's reads of A (4 KB
-// per MMA, 32 cycles: with 16 to 96 columns a tap multiplies no longer than that).
+// sets the error flag.  What bounds a layer is not the MMAs (tensor pipe active 6 to
+// 16 % of the time, 4 images: at 32 cycles to read a 4 KB A operand they need 420 us of 16
+// images) nor any other pipe (none above half): long-scoreboard waits lead, and the
+// operands of a chunk are some 1600 copies of 16 bytes per four rows from four warps.
 // 16 images 256 x 1024, the thirteen 3x3 layers and the head: with one tile per
 // CTA, two to three CTAs per SM and two stages the copies (800 us), MMAs (540) and
 // stores (440) ran one after the other, 2190 us; so 1280 us.  Weights in their own
